@@ -45,6 +45,15 @@ __global__ void __launch_bounds__(352, 3) k_move_z_nodes(const MoveZArgs* nodes,
   move_z_block(a, blockIdx.x, threadIdx.x, blockDim.x);
 }
 
+// The integer form: blockIdx.y = triple, blockIdx.z = node.
+__global__ void __launch_bounds__(256, 4) k_move_z_fixed_nodes(const MoveZArgs* nodes, const int* nblocks) {
+  const MoveZArgs& a = nodes[blockIdx.z];
+  const int w = blockIdx.x * 8 + (threadIdx.x >> 5);
+  if ((int)blockIdx.y * a.n >= nblocks[blockIdx.z] || w >= fixed_warps(a.n)) return;
+  if (!a.sc->have_snap || a.sc->done) return;
+  move_z_fixed_warp(a, blockIdx.y, w, threadIdx.x & 31);
+}
+
 __global__ void __launch_bounds__(512) k_phase2_nodes(const Phase2Args* nodes, const int* nblocks) {
   if ((int)blockIdx.x >= nblocks[blockIdx.y]) return;
   const Phase2Args a = nodes[blockIdx.y];
@@ -166,6 +175,7 @@ struct Wave {
   std::vector<LearnedStart> learned;  // one per node when warm == 2
   int nn = 0;
   int two_phase = 0;
+  int fixed = 1;  // every node's z move takes the integer form
   int cold = 0;  // warm == 0: no LAP of the wave has start duals
   long long total[kStages] = {0, 0, 0, 0};
   int max_m[kStages] = {0, 0, 0, 0};
@@ -244,7 +254,11 @@ cudaError_t enqueue_wave_iteration(const Wave& w, const WaveDev& d, int dual_mod
     k_move_y_nodes<<<dim3(bx, w.nn), 256, 0, s>>>(d.my);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
-  k_move_z_nodes<<<dim3(w.max_blocks, w.nn), move_z_threads(w.max_n), 0, s>>>(d.mz, d.mz_blocks);
+  if (w.fixed)
+    k_move_z_fixed_nodes<<<dim3((fixed_warps(w.max_n) + 7) / 8, w.max_blocks / w.max_n, w.nn), 256, 0, s>>>(
+        d.mz, d.mz_blocks);
+  else
+    k_move_z_nodes<<<dim3(w.max_blocks, w.nn), move_z_threads(w.max_n), 0, s>>>(d.mz, d.mz_blocks);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   for (const LearnedStart& ls : w.learned)
     if ((e = mlp_predict_enqueue(w.mlp, ls.T, ls.m, ls.Dhat, ls.xi, ls.u0, s)) != cudaSuccess) return e;
@@ -358,6 +372,7 @@ void add_node(Wave& w, WaveHost& h, int j, const IterView& v, const rlt2_params&
   }
   h.my[j] = make_move_y(v);
   h.mz[j] = make_move_z(v);
+  w.fixed = w.fixed && h.mz[j].fixed;
   h.p2[j] = make_phase2(v);
   h.mzb[j] = v.ntrip * nr;
   h.fin[j] = make_fin(v);

@@ -6,6 +6,7 @@
 #include <cmath>
 
 #include "rlt2_internal.h"
+#include "rlt2_movefx.cuh"
 
 namespace rlt2 {
 
@@ -182,6 +183,9 @@ struct MoveZArgs {
   int folded;   // S, kz = 1, all phi equal: psi holds psi - tile term, s = (D - xi) - psi,
                 // D' = fma(c1, s, fma(phi, S, D)) with c1 = -(1 + phi)
   double c1;
+  int fixed;        // folded move in integers (canonical duals in fixed point; see rlt2_movefx.cuh)
+  FxFactor phi_fx;  // phi of the fixed form
+  unsigned rcp_groups, rcp_8m;  // ceil(2^31 / d), d = fixed_groups(n) and 8 m: exact quotients while x d < 2^31
   const double* saterm;  // n*n Type 4 amounts (F variant, when sc->sa_on)
   double* Dhat;
   const double* xi;
@@ -275,9 +279,83 @@ __device__ __forceinline__ double ldv(const double* p) {
   else return *p;
 }
 
+// The folded move of the class {(i,p),(j,q),(k,r)}, i < j < k, in the integer
+// form; cr is r's position among the locations without p and q.  Member order
+// and indices are those of RLT2_CLASS_TABLES, written out so that what does not
+// depend on the locations is formed once per block: 32-bit indices (at most
+// 885,657,600 entries for n = 32).
+template <bool RO>
+__device__ __forceinline__ void move_class_fixed(const MoveZArgs& a, int i, int j, int k, int p, int q, int r, int cr) {
+  const unsigned n = a.n, m = a.m, n1 = n - 1, n2 = n1 * n1;
+  const unsigned qp = q > p, rp = r > p, rq = r > q;  // 1 where the first is the larger
+  const unsigned cq = q - qp - (1u - rq), cp = p - (1u - qp) - (1u - rp);
+  // tile (a, la, b, lb) = ((a n + la) (n-1) + b') (n-1) + lb'; row c'', column
+  const unsigned ib = i * n * n2, jb = j * n * n2, kb = k * n * n2;
+  const unsigned t[6] = {ib + (j - 1) * n1 + p * n2 + (q - qp), ib + (k - 1) * n1 + p * n2 + (r - rp),
+                         jb + i * n1 + q * n2 + (p - (1u - qp)), jb + (k - 1) * n1 + q * n2 + (r - rq),
+                         kb + i * n1 + r * n2 + (p - (1u - rp)), kb + j * n1 + r * n2 + (q - (1u - rq))};
+  const unsigned row[6] = {(unsigned)k - 2, (unsigned)j - 1, (unsigned)k - 2, (unsigned)i, (unsigned)j - 1, (unsigned)i};
+  const unsigned col[6] = {(unsigned)cr, cq, (unsigned)cr, cp, cq, cp};
+  double D[6], w[6];
+  unsigned at[6];
+#pragma unroll
+  for (int b = 0; b < 6; ++b) {
+    const unsigned tm = RLT2_IDX(t[b], n * n * n2) * m;
+    at[b] = (tm + RLT2_IDX(row[b], m)) * m + RLT2_IDX(col[b], m);
+    D[b] = a.Dhat[at[b]];
+    w[b] = dadd_(ldv<RO>(a.xi + tm + row[b]), ldv<RO>(a.psi + tm + col[b]));
+  }
+  if (!move_class_fx(D, w, a.phi_fx)) {
+    double s[6], S = 0.0;
+#pragma unroll
+    for (int b = 0; b < 6; ++b) {
+      s[b] = dsub_(D[b], w[b]);
+      S = b ? dadd_(S, s[b]) : s[0];
+    }
+#pragma unroll
+    for (int b = 0; b < 6; ++b) D[b] = __fma_rn(a.c1, s[b], __fma_rn(a.w[0], S, D[b]));
+  }
+#pragma unroll
+  for (int b = 0; b < 6; ++b) a.Dhat[at[b]] = D[b];
+}
+
+// Work of the integer form's launches.  Each of a class's six planes (ordered
+// facility pair, third facility) is contiguous in one of the three locations
+// and a new row for every pair of the other two, so a warp's lanes cover 2 p x
+// 4 q x 4 r: 64 segments of two to four entries for its 192 (32 (q, r) of one p
+// take 144, a band of 8 q x 4 r 96).  The (q, r) of a p run in bands of eight
+// q, r outer, in groups of 32 slots (8 q x 4 r), so that only the last group
+// has idle lanes for any n; the four warps of a group hold its two q halves
+// for two pairs of p, and the two groups of a block the next four r, so that
+// the sectors that a segment shares with its neighbours are read once.
+__host__ __device__ inline int fixed_groups(int n) { return ((n - 1) * (n - 2) + 31) / 32; }
+__host__ __device__ inline int fixed_warps(int n) { return (n + 3) / 4 * fixed_groups(n) * 4; }  // per triple
+
+// Warp w (of fixed_warps) of triple tr.
+__device__ __forceinline__ void move_z_fixed_warp(const MoveZArgs& a, int tr, int w, int lane) {
+  const int n = a.n, m = a.m, n1 = n - 1;
+  const int quad = (int)__umulhi((unsigned)(w >> 2) << 1, a.rcp_groups);  // (w / 4) / fixed_groups
+  const int g = (w >> 2) - quad * fixed_groups(n);
+  const int p = 4 * quad + ((w & 1) << 1) + ((lane >> 2) & 1);
+  const int u = 32 * g + ((lane & 3) << 3 | (w & 2) << 1 | lane >> 3);
+  if (p >= n || u >= n1 * m) return;
+  const int band = (int)__umulhi((unsigned)u << 1, a.rcp_8m);  // u / (8 m)
+  const int cb = u - band * 8 * m, hb = min(8, n1 - 8 * band);
+  const int rr = hb == 8 ? cb >> 3 : cb / hb;
+  const int qq = 8 * band + cb - rr * hb;
+  const int q = qq + (qq >= p);
+  const int lo = p < q ? p : q, hi = p < q ? q : p;
+  int r = rr;
+  r += (r >= lo);
+  r += (r >= hi);
+  const int packed = a.trips[tr];
+  move_class_fixed<true>(a, packed & 255, (packed >> 8) & 255, packed >> 16, p, q, r, rr);
+}
+
 // The classes (q, r) = first, first + stride, ... of block blk = (triple, p);
-// BAND: the banded class order for n >= 22 (see class_of).
-template <bool RO = true, bool BAND = true>
+// BAND: the banded class order for n >= 22 (see class_of).  FIXED: the launch
+// may be asked for the integer form (a.fixed).
+template <bool RO = true, bool BAND = true, bool FIXED = false>
 __device__ __forceinline__ void move_z_block(const MoveZArgs& a, int blk, int first, int stride) {
   if (a.half) {
     move_z_half_block(a, blk);
@@ -299,6 +377,10 @@ __device__ __forceinline__ void move_z_block(const MoveZArgs& a, int blk, int fi
     int r = rr;
     r += (r >= lo);
     r += (r >= hi);
+    if (FIXED && a.fixed) {
+      move_class_fixed<RO>(a, F3[0], F3[1], F3[2], p, q, r, rr);
+      continue;
+    }
     const int L3[3] = {p, q, r};
     double s[6], base[6];
     long long idx[6];
