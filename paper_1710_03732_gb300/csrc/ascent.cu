@@ -314,7 +314,7 @@ static std::mutex g_pool_mu;
 constexpr int kPoolDevices = 64;
 static cudaMemPool_t g_pool[kPoolDevices];
 
-static cudaError_t ctx_pool(cudaMemPool_t* out) {
+cudaError_t rlt2::library_pool(cudaMemPool_t* out) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
@@ -502,7 +502,7 @@ static rlt2_status ctx_alloc(rlt2_ctx* c, bool own_qap) {
                 sizeof(int) * (size_t)(c->ntrip + nr + (prm.half_z ? c->T / 2 : 0)) + (64u << 20);
   size_t fr = 0, tot = 0;
   cudaMemPool_t pool = nullptr;
-  cudaError_t e = ctx_pool(&pool);
+  cudaError_t e = library_pool(&pool);
   if (e == cudaSuccess) e = cudaMemGetInfo(&fr, &tot);
   if (e != cudaSuccess) {
     delete c;

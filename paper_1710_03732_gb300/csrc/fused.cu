@@ -53,8 +53,7 @@ template <int G, bool FX, bool RR = false>
 __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32, 4) k_move_lap_z(MoveZArgs mz, LapArgs a, PipeArgs pa) {
   DevScalars* sc = pa.sc;
   if (sc->done) return;  // stopped: no work, counters untouched
-  using A = typename std::conditional<FX, ArithFx, ArithF64>::type;
-  using T = typename A::T;
+  using T = typename std::conditional<FX, long long, double>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int per = 32 / G;
   const int lane = threadIdx.x & 31;
@@ -132,8 +131,9 @@ __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32, 4) k_move_lap_z(MoveZA
     T u0 = T(0);
     if (warm && live && gl < m) u0 = start_dual<FX>(a.u0[t * m + gl], L);
     __syncwarp();
-    const WarpLapResult<T> R =
-        group_lap<G, true, A, RR && FX>(tile, ld, live ? m : 0, lane, warm, u0, a.dual_mode, scr, uv + grp * G);
+    WarpLapResult<T> R;
+    if constexpr (FX) R = group_lap_fx<G, RR>(tile, ld, live ? m : 0, lane, warm, u0, scr, uv + grp * G);
+    else R = group_lap<G, true>(tile, ld, live ? m : 0, lane, warm, u0, a.dual_mode, scr, uv + grp * G);
     if (live && gl < m) {
       a.u[t * m + gl] = out_value<FX>(R.u, L);
       a.v[t * m + gl] = out_value<FX>(R.v, L);

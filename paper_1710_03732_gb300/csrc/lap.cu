@@ -15,16 +15,95 @@ int default_group(int m) { return m <= 8 ? 8 : (m <= 16 ? 16 : 32); }
 // and start duals are copied into shared memory by cp.async while the current
 // LAP is solved, so the tile's HBM latency is off the warp's path.  The copy
 // of tile k+1 is issued as soon as the column reduction of tile k has
-// converted its raw entries (group_lap's hook); the grid exponent of a tile is
+// converted its raw entries (group_lap_fx's hook); the grid exponent of a tile is
 // the largest exponent field of its raw entries, as in stage_tile.  Results
 // are those of the staged form bit for bit.  With a.head set, warps claim
 // their next step of 32/G LAPs from that counter (zero at launch) when they
 // issue its copies, so that warps whose LAPs needed few searches take more of
 // them and all warps end together; otherwise they take a fixed grid stride.
+template <int PER>
+__device__ __forceinline__ long long claim_step(const LapArgs& a, long long t, int lane) {
+  if (a.head == nullptr || t < a.fixed_part) return t;
+  unsigned long long b = 0;
+  if (lane == 0) b = atomicAdd(a.head, (unsigned long long)PER);
+  return a.fixed_part + (long long)__shfl_sync(kFull, b, 0);
+}
+
+// The same for LAPs whose two tile buffers would leave too few warps on an SM
+// (launch_lap's rule): one tile per warp, converted onto the grid in place.
+// The next tile is only prefetched into L2 while the current one is solved and
+// copied into shared memory after it; the other warps cover that latency.
+template <bool RR>
+__device__ __forceinline__ void k_lap_one_tile(const LapArgs& a, unsigned char* base, int lane, bool warm,
+                                               long long first, long long stride) {
+  using T = long long;
+  constexpr int G = 32;
+  const int m = a.m, ld = tile_ld(m), mm = m * m;
+  T* tile = reinterpret_cast<T*>(base);
+  T* uv = tile + (size_t)m * ld;
+  int* scr = reinterpret_cast<int*>(uv + 32);
+  const double* raw = reinterpret_cast<const double*>(tile);
+  unsigned long long aug_acc = 0, relax_acc = 0;
+  auto slot = [&](long long tb) { return a.map ? (long long)a.map[tb] : tb; };
+  // entries e = lane, lane + 32, ... of the tile, (r, c) advanced without a division per entry
+  const int q32 = 32 / m, r32 = 32 - q32 * m, r_first = lane / m, c_first = lane - r_first * m;
+  for (int r = lane; r < m; r += 32)
+    if (ld > m) tile[r * ld + m] = 0;  // the padding column takes part in the exponent sweep
+  long long t = claim_step<1>(a, first, lane);
+  long long t_static = first;
+  while (t < a.batch) {
+    const long long ts = slot(t);
+    const double* src = a.A + ts * mm;
+    for (int e = lane, r = r_first, c = c_first; e < mm; e += 32) {
+      cp_async8(tile + r * ld + c, src + e);
+      r += q32;
+      c += r32;
+      if (c >= m) {
+        c -= m;
+        ++r;
+      }
+    }
+    cp_async_commit();
+    const double u0d = (warm && lane < m) ? __ldcs(a.u0 + ts * m + lane) : 0.0;
+    cp_async_wait_all();
+    __syncwarp();
+    unsigned eb = 0;
+    for (int e = lane; e < m * ld; e += 32) eb = max(eb, fx_expfield_hi(raw + e));
+    eb = __reduce_max_sync(kFull, eb);
+    const int L = fx_grid(eb);
+    const T u0 = (warm && lane < m) ? start_dual<true>(u0d, L) : T(0);
+    long long next = a.batch;
+    const WarpLapResult<T> R = group_lap_fx<G, RR>(tile, ld, m, lane, warm, u0, scr, uv, raw, ld, L, [&]() {
+      t_static += stride;
+      next = claim_step<1>(a, t_static, lane);
+      if (next < a.batch) {
+        const char* p = reinterpret_cast<const char*>(a.A + slot(next) * mm);
+        for (int o = lane * 128; o < mm * 8; o += 32 * 128) asm volatile("prefetch.global.L2 [%0];" ::"l"(p + o));
+      }
+    });
+    if (lane < m) {
+      if (a.u) a.u[ts * m + lane] = out_value<true>(R.u, L);
+      if (a.v) a.v[ts * m + lane] = out_value<true>(R.v, L);
+      if (a.r2c) a.r2c[ts * m + lane] = R.r2c;
+    }
+    if (lane == 0) {
+      a.value[ts] = out_value<true>(R.value, L);
+      if (a.naug) a.naug[ts] = R.naug;
+      aug_acc += R.naug;
+      relax_acc += R.nrelax;
+    }
+    __syncwarp();
+    t = next;
+  }
+  if (a.stats && lane == 0 && (aug_acc | relax_acc)) {
+    atomicAdd(a.stats + 0, aug_acc);
+    atomicAdd(a.stats + 1, relax_acc);
+  }
+}
+
 template <int G, bool RR>
 __device__ __forceinline__ void k_lap_prefetching(const LapArgs& a, unsigned char* base, int lane, bool warm,
                                                   long long first, long long stride) {
-  using A = ArithFx;
   using T = long long;
   constexpr int per = 32 / G;
   const int grp = lane / G, gl = lane & (G - 1);
@@ -45,14 +124,11 @@ __device__ __forceinline__ void k_lap_prefetching(const LapArgs& a, unsigned cha
     }
     cp_async_commit();
   };
-  // the first LAP of this warp's next step (every lane of the warp)
-  auto claim = [&](long long t_static) -> long long {
-    if (a.head == nullptr) return t_static;
-    unsigned long long b = 0;
-    if (lane == 0) b = atomicAdd(a.head, (unsigned long long)per);
-    return (long long)__shfl_sync(kFull, b, 0);
-  };
+  // the first LAP of this warp's next step (every lane of the warp); t = the
+  // step's place in the fixed stride
+  auto claim = [&](long long t) -> long long { return claim_step<per>(a, t, lane); };
   long long t0 = claim(first);
+  long long t_static = first;
   issue(t0);
   while (t0 < a.batch) {
     const long long tb = t0 + grp;
@@ -72,12 +148,13 @@ __device__ __forceinline__ void k_lap_prefetching(const LapArgs& a, unsigned cha
     const int L = fx_grid(eb);
     T u0 = T(0);
     if (warm && have && gl < m) u0 = start_dual<true>(raw[mm + gl], L);
-    long long next = a.batch;  // claimed in the hook, which group_lap calls once (raw is set)
-    const WarpLapResult<T> R = group_lap<G, true, A, RR>(tile, ld, have ? m : 0, lane, warm, u0, a.dual_mode, scr,
-                                                     uv + grp * G, raw, L, [&]() {
-                                                       next = claim(t0 + stride);
-                                                       issue(next);
-                                                     });
+    long long next = a.batch;  // claimed in the hook, which group_lap_fx calls once (raw is set)
+    const WarpLapResult<T> R = group_lap_fx<G, RR>(tile, ld, have ? m : 0, lane, warm, u0, scr, uv + grp * G, raw, m,
+                                                   L, [&]() {
+                                                     t_static += stride;
+                                                     next = claim(t_static);
+                                                     issue(next);
+                                                   });
     if (have && gl < m) {
       if (a.u) a.u[t * m + gl] = out_value<true>(R.u, L);
       if (a.v) a.v[t * m + gl] = out_value<true>(R.v, L);
@@ -99,20 +176,32 @@ __device__ __forceinline__ void k_lap_prefetching(const LapArgs& a, unsigned cha
   }
 }
 
+// Resident blocks that the registers are cut for.  G = 32: four (64 registers)
+// against three (77): Z stage at n = 20 370 against 399 us, n = 30 3.38 against
+// 3.65 ms; G = 16: three against four: n = 12 34.0 against 39.5 us.
+template <int G>
+constexpr int kLapBlocks = G == 16 ? 3 : 4;
+
 // Grid-stride over LAPs, 32/G LAPs per warp per step.  FX selects the exact
 // fixed-point arithmetic (canonical duals), else FP64; RR (fixed point, cold
 // launches) reduces the rows of a cold start first.
 template <int G, bool PRE, bool FX, bool RR = false>
-__global__ void __launch_bounds__(kMaxWarpsPerBlock * 32) k_lap(LapArgs a) {
+__global__ void __launch_bounds__(kMaxWarpsPerBlock * 32, kLapBlocks<G>) k_lap(LapArgs a) {
   if (a.skip && *a.skip) return;
-  using A = typename std::conditional<FX, ArithFx, ArithF64>::type;
-  using T = typename A::T;
+  using T = typename std::conditional<FX, long long, double>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if constexpr (FX && PRE) {
     if (a.prefetch) {
       const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, wpb = blockDim.x >> 5;
       const bool warm = a.u0 != nullptr && (a.warm_gate == nullptr || *a.warm_gate != 0);
       const long long nwarps = (long long)gridDim.x * wpb;
+      if constexpr (G == 32) {
+        if (a.prefetch == 2) {
+          k_lap_one_tile<RR>(a, smem_raw + (size_t)wib * warp_smem_bytes_one(a.m), lane, warm,
+                             (long long)blockIdx.x * wpb + wib, nwarps);
+          return;
+        }
+      }
       k_lap_prefetching<G, RR>(a, smem_raw + (size_t)wib * warp_smem_bytes_async(a.m, G), lane, warm,
                            ((long long)blockIdx.x * wpb + wib) * (32 / G), nwarps * (32 / G));
       return;
@@ -146,8 +235,9 @@ __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32) k_lap(LapArgs a) {
     if (warm && have && gl < m) u0 = start_dual<FX>(a.u0[t * m + gl], L);
     __syncwarp();
     // without a reduced-cost output (PRE) the tile may be overwritten by the canonical pass
-    const WarpLapResult<T> R =
-        group_lap<G, PRE, A, RR && FX>(tile, ld, have ? m : 0, lane, warm, u0, a.dual_mode, scr, uv + grp * G);
+    WarpLapResult<T> R;
+    if constexpr (FX) R = group_lap_fx<G, RR>(tile, ld, have ? m : 0, lane, warm, u0, scr, uv + grp * G);
+    else R = group_lap<G, PRE>(tile, ld, have ? m : 0, lane, warm, u0, a.dual_mode, scr, uv + grp * G);
     if (have && gl < m) {
       if (a.u) a.u[t * m + gl] = out_value<FX>(R.u, L);
       if (a.v) a.v[t * m + gl] = out_value<FX>(R.v, L);
@@ -170,7 +260,7 @@ __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32) k_lap(LapArgs a) {
 #pragma unroll 4
         for (int e = gl; e < mm; e += G) {
           const int r = e / m, c = e - r * m;
-          dst[e] = out_value<FX>(A::sub(A::sub(tile[r * ld + c], ug[r]), vg[c]), L);
+          dst[e] = out_value<FX>(lap_sub(lap_sub(tile[r * ld + c], ug[r]), vg[c]), L);
         }
       }
     }
@@ -180,34 +270,6 @@ __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32) k_lap(LapArgs a) {
     atomicAdd(a.stats + 0, aug_acc);
     atomicAdd(a.stats + 1, relax_acc);
   }
-}
-
-// Launch configuration (SM count, occupancy per size, shared-memory
-// attributes), kept per device and set once per (device, size, group, warps)
-// under g_cfg_mu: contexts may be created and used from different host threads
-// and on different devices.  Like every per-device cache of the library it is
-// not valid across a cudaDeviceReset.
-static std::mutex g_cfg_mu;
-constexpr int kMaxCfgDevices = 64;
-struct LapDevCfg {
-  int sms = 0;                 // multiprocessors of the device
-  int occ[33][3][2] = {};      // blocks per SM for (m, G, warps per block), 0 = not configured
-  int occ_nodes[33][3][2] = {};
-  bool attr[3] = {};           // dynamic shared-memory attribute set (k_lap, per G)
-  bool attr_nodes[3] = {};     // the same for k_lap_nodes
-};
-static LapDevCfg g_devcfg[kMaxCfgDevices];
-
-// The current device's entry, its SM count read on first use (g_cfg_mu held).
-static cudaError_t current_cfg(LapDevCfg** out) {
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (dev < 0 || dev >= kMaxCfgDevices) return cudaErrorInvalidDevice;
-  LapDevCfg& c = g_devcfg[dev];
-  if (!c.sms && (e = cudaDeviceGetAttribute(&c.sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  *out = &c;
-  return cudaSuccess;
 }
 
 static int gidx(int G) { return G == 8 ? 0 : (G == 16 ? 1 : 2); }
@@ -226,36 +288,90 @@ static LapKernel lap_kernel(int G, bool pre, bool fx, bool rr) {
   return G == 8 ? lap_kernel<8>(pre, fx, rr) : (G == 16 ? lap_kernel<16>(pre, fx, rr) : lap_kernel<32>(pre, fx, rr));
 }
 
-// Occupancy of the slowest of the six forms, so that one grid size serves all.
-static cudaError_t prepare_one(LapDevCfg& cfg, int G, int m, int wpb) {
-  int& slot = cfg.occ[m][gidx(G)][wpb == 4 ? 0 : 1];
-  if (slot > 0) return cudaSuccess;
-  bool* attr_set = cfg.attr;
-  cudaError_t e;
-  const int cap = (int)(warp_smem_bytes_async(32, 32) * kMaxWarpsPerBlock);
-  int occ = 1 << 20;
-  for (int k = 0; k < 6; ++k) {
-    const bool pre = (k & 1) != 0, fx = (k & 2) != 0 || k >= 4, rr = k >= 4;
-    const LapKernel kern = lap_kernel(G, pre, fx, rr);
-    if (!attr_set[gidx(G)]) {
-      if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, cap)) != cudaSuccess)
-        return e;
-    }
-    int o = 0;
-    // the prefetching form (fixed point, no reduced-cost output) needs more shared memory
-    const size_t per_warp = (pre && fx) ? warp_smem_bytes_async(m, G) : warp_smem_bytes(m, G);
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, kern, wpb * 32, per_warp * wpb);
-    if (e != cudaSuccess) return e;
-    occ = o < occ ? o : occ;
-  }
-  attr_set[gidx(G)] = true;
-  slot = occ < 1 ? 1 : occ;
+// The forms of k_lap: (pre, fx, rr) and, for the prefetching ones (fixed point,
+// no reduced-cost output), how the tile gets into shared memory.
+constexpr int kForms = 6;
+struct LapForm {
+  bool pre, fx, rr;
+};
+static LapForm lap_form(int k) { return LapForm{(k & 1) != 0, k >= 2, k >= 4}; }
+static int lap_form_index(bool pre, bool fx, bool rr) { return (rr ? 4 : (fx ? 2 : 0)) + (pre ? 1 : 0); }
+
+// A launch of one form on the current device: its resident blocks and, for the
+// prefetching forms, a.prefetch (1 two tile buffers per warp, 2 the one-tile form).
+struct LapPlan {
+  int occ = 0;  // resident blocks per SM, 0 = not configured
+  int prefetch = 0;
+  size_t smem = 0;
+};
+
+// Launch configuration, kept per device and set once per (device, size, group,
+// warps) under g_cfg_mu: contexts may be created and used from different host
+// threads and on different devices.  Like every per-device cache of the library
+// it is not valid across a cudaDeviceReset.
+static std::mutex g_cfg_mu;
+constexpr int kMaxCfgDevices = 64;
+struct LapDevCfg {
+  int sms = 0;                        // multiprocessors of the device
+  LapPlan plan[33][3][2][kForms];     // for (m, G, warps per block, form)
+  int occ_nodes[33][3][2] = {};
+  bool attr[3] = {};                  // dynamic shared-memory attribute set (k_lap, per G)
+  bool attr_nodes[3] = {};            // the same for k_lap_nodes
+};
+static LapDevCfg g_devcfg[kMaxCfgDevices];
+
+// The current device's entry, its SM count read on first use (g_cfg_mu held).
+static cudaError_t current_cfg(LapDevCfg** out) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= kMaxCfgDevices) return cudaErrorInvalidDevice;
+  LapDevCfg& c = g_devcfg[dev];
+  if (!c.sms && (e = cudaDeviceGetAttribute(&c.sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+  *out = &c;
   return cudaSuccess;
 }
 
-// Configures (once per device) the launch of an m-column LAP; *cap (nullable)
-// receives the resident block count of that launch on the current device.
-static cudaError_t prepare_cap(int m, int group, int warps_per_block, long long* cap) {
+// Every form of (G, m, wpb).  A prefetching form takes two tile buffers per
+// warp unless one tile alone lets more warps onto an SM: m = 28 (16 -> 32
+// warps), not m = 18 (32 either way).
+static cudaError_t prepare_one(LapDevCfg& cfg, int G, int m, int wpb) {
+  LapPlan* plan = cfg.plan[m][gidx(G)][wpb == 4 ? 0 : 1];
+  if (plan[kForms - 1].occ > 0) return cudaSuccess;
+  cudaError_t e;
+  const int cap = (int)(warp_smem_bytes_async(32, 32) * kMaxWarpsPerBlock);
+  for (int k = 0; k < kForms; ++k) {
+    const LapForm f = lap_form(k);
+    const LapKernel kern = lap_kernel(G, f.pre, f.fx, f.rr);
+    if (!cfg.attr[gidx(G)] &&
+        (e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, cap)) != cudaSuccess)
+      return e;
+    auto occupancy = [&](size_t per_warp, int* o) {
+      return cudaOccupancyMaxActiveBlocksPerMultiprocessor(o, kern, wpb * 32, per_warp * wpb);
+    };
+    LapPlan p;
+    p.prefetch = f.pre && f.fx ? 1 : 0;
+    p.smem = (p.prefetch ? warp_smem_bytes_async(m, G) : warp_smem_bytes(m, G)) * wpb;
+    if ((e = occupancy(p.smem / wpb, &p.occ)) != cudaSuccess) return e;
+    if (p.prefetch && G == 32) {
+      int one = 0;
+      if ((e = occupancy(warp_smem_bytes_one(m), &one)) != cudaSuccess) return e;
+      if (one > p.occ) {
+        p.occ = one;
+        p.prefetch = 2;
+        p.smem = warp_smem_bytes_one(m) * wpb;
+      }
+    }
+    if (p.occ < 1) p.occ = 1;
+    plan[k] = p;
+  }
+  cfg.attr[gidx(G)] = true;
+  return cudaSuccess;
+}
+
+// The plan of an m-column LAP launch on the current device (configured on
+// first use), *cap its resident block count.
+static cudaError_t prepare_plan(int m, int group, int warps_per_block, int form, LapPlan* plan, long long* cap) {
   if (m < 1 || m > 32) return cudaErrorInvalidValue;
   const int G = group ? group : default_group(m);
   const int wpb = warps_per_block ? warps_per_block : kMaxWarpsPerBlock;
@@ -265,34 +381,52 @@ static cudaError_t prepare_cap(int m, int group, int warps_per_block, long long*
   cudaError_t e = current_cfg(&cfg);
   if (e != cudaSuccess) return e;
   if ((e = prepare_one(*cfg, G, m, wpb)) != cudaSuccess) return e;
-  if (cap) *cap = (long long)cfg->sms * cfg->occ[m][gidx(G)][wpb == 4 ? 0 : 1];
+  *plan = cfg->plan[m][gidx(G)][wpb == 4 ? 0 : 1][form];
+  *cap = (long long)cfg->sms * plan->occ;
   return cudaSuccess;
 }
 
 cudaError_t prepare_lap(int m, int group, int warps_per_block) {
-  return prepare_cap(m, group, warps_per_block, nullptr);
+  LapPlan plan;
+  long long cap = 0;
+  return prepare_plan(m, group, warps_per_block, 0, &plan, &cap);
 }
 
 cudaError_t launch_lap(const LapArgs& a, cudaStream_t s) {
   if (a.batch <= 0) return cudaSuccess;
   const int G = a.group ? a.group : default_group(a.m);
   const int wpb = a.warps_per_block ? a.warps_per_block : kMaxWarpsPerBlock;
+  // a cold fixed-point launch reduces the rows first (the same canonical result)
+  const bool pre = a.pi == nullptr && a.Badd == nullptr, fx = a.dual_mode == 1, rr = fx && a.u0 == nullptr;
+  LapPlan plan;
   long long cap = 0;
-  cudaError_t e = prepare_cap(a.m, G, wpb, &cap);
+  cudaError_t e = prepare_plan(a.m, G, wpb, lap_form_index(pre, fx, rr), &plan, &cap);
   if (e != cudaSuccess) return e;
   LapArgs b = a;
-  b.prefetch = (a.dual_mode == 1 && a.pi == nullptr && a.Badd == nullptr) ? 1 : 0;
-  const size_t smem = (b.prefetch ? warp_smem_bytes_async(a.m, G) : warp_smem_bytes(a.m, G)) * wpb;
+  b.prefetch = plan.prefetch;
   const long long per_block = (long long)wpb * (32 / G);
   const long long need = (a.batch + per_block - 1) / per_block;
   const int grid = (int)(need < cap ? need : cap);
-  // a cold fixed-point launch reduces the rows first (the same canonical result)
-  const LapKernel kern = lap_kernel(G, a.pi == nullptr, a.dual_mode == 1, a.dual_mode == 1 && a.u0 == nullptr);
-  if (!b.prefetch) b.head = nullptr;
-  if (b.head && !b.head_zeroed && (e = cudaMemsetAsync(b.head, 0, sizeof(unsigned long long), s)) != cudaSuccess)
-    return e;
-  kern<<<grid, wpb * 32, smem, s>>>(b);
+  if (!b.prefetch || need <= cap) b.head = nullptr;  // one step per warp: nothing to share out
+  if (b.head) {
+    // half of the steps by fixed stride, the rest from the queue, so that the
+    // warps still end together: the counter is one address, and at n = 20 the
+    // 144,400 claims alone take 160 us (Z stage: none by stride 374 us, half 370,
+    // three quarters 397)
+    const long long round = (long long)grid * per_block;
+    b.fixed_part = a.batch / round / 2 * round;
+    if (!b.head_zeroed && (e = cudaMemsetAsync(b.head, 0, sizeof(unsigned long long), s)) != cudaSuccess) return e;
+  }
+  lap_kernel(G, pre, fx, rr)<<<grid, wpb * 32, plan.smem, s>>>(b);
   return cudaGetLastError();
+}
+
+bool lap_wants_queue(long long batch, int m) {
+  LapPlan plan;
+  long long cap = 0;
+  const int G = default_group(m);
+  if (prepare_plan(m, G, kMaxWarpsPerBlock, lap_form_index(true, true, false), &plan, &cap) != cudaSuccess) return false;
+  return batch > cap * kMaxWarpsPerBlock * (32 / G);
 }
 
 // ---------------------------------------------------------------------------
@@ -302,13 +436,12 @@ cudaError_t launch_lap(const LapArgs& a, cudaStream_t s) {
 // The queue-fed node form of k_lap_prefetching (fixed point, Z stages): a
 // warp claims its next queue slot before it solves the current one and copies
 // that slot's tiles and start duals into shared memory by cp.async (issued by
-// group_lap's hook once the current raw tiles are converted).  The raw buffers
+// group_lap_fx's hook once the current raw tiles are converted).  The raw buffers
 // are sized for the largest LAP of the stage.  Results are those of the staged
 // form bit for bit (each LAP is independent of which warp solves it).
 template <int G, bool RR>
 __device__ __forceinline__ void k_lap_nodes_prefetching(const NodeLapArgs& a, const long long* s_prefix,
                                                         unsigned char* base, int lane) {
-  using A = ArithFx;
   using T = long long;
   constexpr int per = 32 / G;
   const int grp = lane / G, gl = lane & (G - 1);
@@ -378,8 +511,8 @@ __device__ __forceinline__ void k_lap_nodes_prefetching(const NodeLapArgs& a, co
     }
     const int L = fx_grid(eb);
     const T u0 = (cur.warm && gl < m) ? start_dual<true>(raw[mm + gl], L) : T(0);
-    const WarpLapResult<T> R = group_lap<G, true, A, RR>(tile, tile_ld(m), m, lane, cur.warm, u0, a.dual_mode, scr,
-                                                     uv + grp * G, raw, L, [&]() { issue(nxt); });
+    const WarpLapResult<T> R = group_lap_fx<G, RR>(tile, tile_ld(m), m, lane, cur.warm, u0, scr, uv + grp * G, raw, m,
+                                                   L, [&]() { issue(nxt); });
     if (cur.have) {
       const NodeLapItem& it = a.items[cur.k];
       if (gl < m) {
@@ -406,8 +539,7 @@ __device__ __forceinline__ void k_lap_nodes_prefetching(const NodeLapArgs& a, co
 
 template <int G, bool PRE, bool FX, bool RR = false>
 __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32) k_lap_nodes(NodeLapArgs a) {
-  using A = typename std::conditional<FX, ArithFx, ArithF64>::type;
-  using T = typename A::T;
+  using T = typename std::conditional<FX, long long, double>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int per = 32 / G;
   long long* s_prefix = reinterpret_cast<long long*>(smem_raw);
@@ -462,8 +594,9 @@ __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32) k_lap_nodes(NodeLapArg
     const bool warm = have && it.u0 != nullptr && (it.warm_gate == nullptr || *it.warm_gate != 0);
     const T u0 = (warm && gl < m) ? start_dual<FX>(it.u0[li * m + gl], L) : T(0);
     __syncwarp();
-    const WarpLapResult<T> R =
-        group_lap<G, PRE, A, RR && FX>(tile, ld, m, lane, warm, u0, a.dual_mode, scr, uv + grp * G);
+    WarpLapResult<T> R;
+    if constexpr (FX) R = group_lap_fx<G, RR>(tile, ld, m, lane, warm, u0, scr, uv + grp * G);
+    else R = group_lap<G, PRE>(tile, ld, m, lane, warm, u0, a.dual_mode, scr, uv + grp * G);
     if (have && gl < m) {
       if (it.u) it.u[li * m + gl] = out_value<FX>(R.u, L);
       if (it.v) it.v[li * m + gl] = out_value<FX>(R.v, L);
@@ -483,7 +616,7 @@ __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32) k_lap_nodes(NodeLapArg
       const T* vg = uv + 32 + grp * G;
       for (int e = gl; e < mm; e += G) {
         const int r = e / m, c = e - r * m;
-        dst[e] = out_value<FX>(A::sub(A::sub(tile[r * ld + c], ug[r]), vg[c]), L);
+        dst[e] = out_value<FX>(lap_sub(lap_sub(tile[r * ld + c], ug[r]), vg[c]), L);
       }
     }
     __syncwarp();
@@ -584,12 +717,21 @@ extern "C" rlt2_status rlt2_lap_batched(int batch, int m, const double* cost, co
   a.naug = n_aug;
   a.dual_mode = dual_mode;
   const cudaStream_t s = (cudaStream_t)stream;
-  // the fixed-point form's LAP queue: 8 stream-ordered bytes, freed after the launch
-  // (without them the warps take a fixed stride; the results are the same)
+  // the fixed-point form's LAP queue: 8 stream-ordered bytes of the library's
+  // pool, freed after the launch (without them the warps take a fixed stride;
+  // the results are the same).  A batch that the resident warps hold at once
+  // needs none
   unsigned long long* head = nullptr;
-  if (dual_mode == 1 && cudaMallocAsync((void**)&head, sizeof(unsigned long long), s) != cudaSuccess) {
+  if (dual_mode == 1 && lap_wants_queue(batch, m)) {
+    // under stream capture the pool may not be created: the default one then
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    cudaMemPool_t pool = nullptr;
+    const bool own = cudaStreamIsCapturing(s, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone &&
+                     library_pool(&pool) == cudaSuccess;
+    const cudaError_t ea = own ? cudaMallocFromPoolAsync((void**)&head, sizeof(unsigned long long), pool, s)
+                               : cudaMallocAsync((void**)&head, sizeof(unsigned long long), s);
+    if (ea != cudaSuccess) head = nullptr;
     (void)cudaGetLastError();
-    head = nullptr;
   }
   a.head = head;
   cudaError_t e = launch_lap(a, s);

@@ -65,7 +65,8 @@ struct LapArgs {
   int group;                 // lanes per LAP (8, 16 or 32); 0 = smallest that fits m
   int warps_per_block;       // 4 or 8; 0 = 8
   const int* map;            // nullable: LAP b works on slot map[b] of every array (a subset of tiles)
-  int prefetch;              // set by launch_lap: the fixed-point form without Badd and pi stages
+  long long fixed_part;      // set by launch_lap: LAPs below this are taken in a fixed stride, the rest from head
+  int prefetch;              // set by launch_lap (2: its one-tile form): the fixed-point form without Badd and pi stages
                              // the next tile by cp.async while it solves the current one
   unsigned long long* head;  // nullable: device counter of the prefetching form's LAP queue
                              // (launch_lap zeroes it on the stream before the launch)
@@ -151,6 +152,13 @@ cudaError_t prepare_lap(int m, int group = 0, int warps_per_block = 0);
 
 // Enqueue the batched LAP kernel (grid sized for the device); returns the CUDA error.
 cudaError_t launch_lap(const LapArgs& a, cudaStream_t s);
+
+// Whether a fixed-point batch of the default shape is more than its resident
+// warps hold at once, so that launch_lap would use a queue (LapArgs::head).
+bool lap_wants_queue(long long batch, int m);
+
+// The library's stream-ordered memory pool on the current device (ascent.cu).
+cudaError_t library_pool(cudaMemPool_t* out);
 
 constexpr int kRing = 1 << 16;  // bound-history ring (entries)
 

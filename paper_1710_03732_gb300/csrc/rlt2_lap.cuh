@@ -93,25 +93,6 @@ __device__ __forceinline__ int warp_argmin(unsigned long long key) {
 __device__ __forceinline__ double dsub(double a, double b) { return __dsub_rn(a, b); }
 __device__ __forceinline__ double dadd(double a, double b) { return __dadd_rn(a, b); }
 
-// Arithmetic of group_lap: value type, subtraction, addition and an
-// order-preserving unsigned key.
-struct ArithF64 {
-  using T = double;
-  static constexpr bool kExact = false;  // rounded: keys are cached next to the values
-  static __device__ __forceinline__ T sub(T a, T b) { return __dsub_rn(a, b); }
-  static __device__ __forceinline__ T add(T a, T b) { return __dadd_rn(a, b); }
-  static __device__ __forceinline__ unsigned long long key(T x) { return okey(x); }
-};
-struct ArithFx {
-  using T = long long;
-  static constexpr bool kExact = true;  // exact: keys are the values with the sign bit flipped
-  static __device__ __forceinline__ T sub(T a, T b) { return a - b; }
-  static __device__ __forceinline__ T add(T a, T b) { return a + b; }
-  static __device__ __forceinline__ unsigned long long key(T x) {
-    return (unsigned long long)x ^ 0x8000000000000000ull;
-  }
-};
-
 // ---- fixed-point grid of a tile -------------------------------------------
 // Biased exponent field of a double (0 for zeros and subnormals).
 __device__ __forceinline__ unsigned fx_expfield(double x) {
@@ -131,17 +112,6 @@ __device__ __forceinline__ long long fx_floor(double x, int L, int lim) {
   const int e = (eb ? eb : 1) - 1075;  // |x| = mant * 2^e
   if (e + 53 - L > lim) return b < 0 ? -(1ll << lim) : (1ll << lim);
   const int sh = min(L - e, 63);       // >= 53 - lim > 0
-  return (b < 0 ? -mant : mant) >> sh;
-}
-
-// fx_floor for an entry of the tile whose grid is L: its exponent is at most
-// the tile's largest, so |x| < 2^(L + 48) and the clamp of fx_floor cannot
-// apply; the result is the same.
-__device__ __forceinline__ long long fx_floor_entry(double x, int L) {
-  const long long b = __double_as_longlong(x);
-  const int eb = (int)((b >> 52) & 0x7ff);
-  const long long mant = (b & 0xFFFFFFFFFFFFFll) | (eb ? (1ll << 52) : 0ll);
-  const int sh = min(L + 1075 - (eb ? eb : 1), 63);  // >= 5
   return (b < 0 ? -mant : mant) >> sh;
 }
 
@@ -226,116 +196,47 @@ __device__ __forceinline__ unsigned group_bits(unsigned ball, int gb) {
   else return (ball >> gb) & ((1u << G) - 1u);
 }
 
-// Called by group_lap once the column reduction has read the staged raw tile
+// Called by group_lap_fx once the column reduction has read the staged raw tile
 // (all lanes, after a __syncwarp): the caller may then reuse the raw buffer.
 struct NoHook {
   __device__ __forceinline__ void operator()() const {}
 };
 
-// Solve one LAP per group of G lanes (32/G LAPs per warp) in lockstep: every
-// intrinsic is executed by all 32 lanes with the full mask and all loops are
-// warp-uniform (they run while any group still has work; idle groups only
-// predicate their updates), so the LAPs of one warp share every instruction.
-// Group lane gl = lane % G holds row gl and column gl of its LAP.  `cs` is the
-// group's m x m tile (row stride ld) in shared memory, `scr` G ints of group
-// scratch, m the group's LAP size (0 = no LAP, 1 <= m <= G otherwise).  The
-// arithmetic is identical for every G.
+// Solve one LAP per group of G lanes (32/G LAPs per warp) in lockstep, FP64 in
+// the oracle's operation order: every intrinsic is executed by all 32 lanes
+// with the full mask and all loops are warp-uniform (they run while any group
+// still has work; idle groups only predicate their updates), so the LAPs of
+// one warp share every instruction.  Group lane gl = lane % G holds row gl and
+// column gl of its LAP.  `cs` is the group's m x m tile (row stride ld) in
+// shared memory, `scr` G ints of group scratch, m the group's LAP size (0 = no
+// LAP, 1 <= m <= G otherwise).  The arithmetic is identical for every G.
 // PRE: the caller does not need the tile afterwards, so the canonical pass may
 // replace it by its reduced costs first (uvs: 64 values of group staging).
-// A: ArithF64 or ArithFx (the tile and u0 already on the grid).
-// raw (fixed point only, nullable): the group's tile as m*m doubles, row-major
-// and unconverted, in shared memory; the column reduction then converts each
-// entry onto the grid 2^L as it reads it (lanes = columns) and stores it into
-// cs, and calls hook() once raw is no longer needed.  Without raw, cs already
-// holds the converted tile.
-// RR (exact form only): a cold start reduces the rows first, u_r = the row's
-// minimum, as the classical Hungarian method does, before the column
-// reduction: fewer searches are left after the greedy matching, and the
-// canonical result does not depend on the start.
-template <int G, bool PRE, typename A, bool RR = false, typename Hook = NoHook>
-__device__ __forceinline__ WarpLapResult<typename A::T> group_lap(typename A::T* __restrict__ cs, int ld, int m,
-                                                                  int lane, bool warm, typename A::T u0,
-                                                                  int dual_mode, int* scr, typename A::T* uvs,
-                                                                  const double* raw = nullptr, int L = 0,
-                                                                  const Hook& hook = Hook()) {
-  using T = typename A::T;
+template <int G, bool PRE>
+__device__ __forceinline__ WarpLapResult<double> group_lap(double* __restrict__ cs, int ld, int m, int lane, bool warm,
+                                                           double u0, int dual_mode, int* scr, double* uvs) {
   const int gl = lane & (G - 1);
   const int gb = lane - gl;
   const bool cv = gl < m;
   const int M = (G == 32) ? m : (int)__reduce_max_sync(kFull, (unsigned)m);
-  WarpLapResult<T> R;
-  T u = (cv && warm) ? u0 : T(0);
-  T v = T(0);
+  WarpLapResult<double> R;
+  double u = (cv && warm) ? u0 : 0.0;
+  double v = 0.0;
   int naug = 0, nrelax = 0;
 
-  // column reduction with the argmin row (fixed point: the row duals are
-  // broadcast from shared memory, one load instead of two shuffles per row;
-  // uvs holds the group's row duals until the canonical pass)
+  // column reduction with the argmin row
   unsigned long long bestk = ~0ull;
   int arg = -1;
-  // exact form: the running minimum starts above every |x| < 2^58, so the first
-  // row always takes it (the same result as testing arg < 0)
-  T vmin = A::kExact ? T(0x7fffffffffffffffll) : T(0);
-  if constexpr (A::kExact && RR) {
-    // warp-uniform (the launches that take RR start every LAP cold)
-    if (!__any_sync(kFull, warm)) {
-      if (raw) {  // the tile onto the grid first (lanes = columns)
-        for (int r = 0; r < M; ++r)
-          if (cv && r < m) cs[r * ld + gl] = fx_floor_entry(raw[r * m + gl], L);
-        __syncwarp();
-        hook();
-        raw = nullptr;
-      }
-      T mn = T(0x7fffffffffffffffll);  // above every entry (|x| < 2^58)
-      for (int c = 0; c < M; ++c)
-        if (cv && c < m) {
-          const T x = cs[gl * ld + c];  // lane = row (odd row stride: no bank conflicts)
-          mn = x < mn ? x : mn;
-        }
-      u = cv ? mn : T(0);
-      warm = true;  // the column reduction below subtracts these row duals
-    }
-  }
-  if constexpr (A::kExact) {
-    uvs[gl] = u;
-    __syncwarp();
-  }
   for (int r = 0; r < M; ++r) {
-    T ur;
-    if constexpr (A::kExact) ur = warm ? uvs[r] : T(0);
-    else ur = __shfl_sync(kFull, u, gb + r);
+    const double ur = __shfl_sync(kFull, u, gb + r);
     if (cv && r < m) {
-      T c;
-      if constexpr (A::kExact) {
-        if (raw) {
-          c = fx_floor_entry(raw[r * m + gl], L);
-          cs[r * ld + gl] = c;
-        } else {
-          c = cs[r * ld + gl];
-        }
-      } else {
-        c = cs[r * ld + gl];
-      }
-      const T x = warm ? A::sub(c, ur) : c;  // c - 0 == c exactly
-      if constexpr (A::kExact) {
-        if (x < vmin) {
-          arg = r;
-          vmin = x;
-        }
-      } else if (arg < 0 || A::key(x) < bestk) {
-        bestk = A::key(x);
+      const double c = cs[r * ld + gl];
+      const double x = warm ? dsub(c, ur) : c;  // c - 0 == c exactly
+      if (arg < 0 || okey(x) < bestk) {
+        bestk = okey(x);
         arg = r;
         v = x;
       }
-    }
-  }
-  if constexpr (A::kExact) {
-    if (cv) v = vmin;
-  }
-  if constexpr (A::kExact) {
-    if (raw) {
-      __syncwarp();  // every lane's reads of raw are done
-      hook();
     }
   }
   // greedy: the lowest column among those sharing an argmin row takes it
@@ -361,19 +262,17 @@ __device__ __forceinline__ WarpLapResult<typename A::T> group_lap(typename A::T*
       ++naug;
       nrelax += m;
     }
-    T ui;
-    if constexpr (A::kExact) ui = uvs[i];
-    else ui = __shfl_sync(kFull, u, gb + i);
-    T d = (act && cv) ? A::sub(A::sub(cs[i * ld + gl], ui), v) : T(0);
-    unsigned long long dk = A::key(d);  // cached key of d (rounded form only)
+    const double ui = __shfl_sync(kFull, u, gb + i);
+    double d = (act && cv) ? dsub(dsub(cs[i * ld + gl], ui), v) : 0.0;
+    unsigned long long dk = okey(d);  // cached key of d
     int pred = i;
     bool scanned = !(act && cv);
     bool searching = act;
     int sink = 0;
-    T dlast = T(0);
+    double dlast = 0.0;
     while (G == 32 ? searching : __any_sync(kFull, searching)) {
-      const int c = group_argmin<G>(scanned ? ~0ull : (A::kExact ? A::key(d) : dk), gb);
-      const T dm = __shfl_sync(kFull, d, gb + c);
+      const int c = group_argmin<G>(scanned ? ~0ull : dk, gb);
+      const double dm = __shfl_sync(kFull, d, gb + c);
       if (searching && gl == c) scanned = true;
       // the matching does not change during a search, so column c is free
       // exactly when it has no matched row
@@ -385,14 +284,12 @@ __device__ __forceinline__ WarpLapResult<typename A::T> group_lap(typename A::T*
       }
       const bool relaxing = searching && !found;
       const int r = r0 < 0 ? 0 : r0;
-      T ur;
-      if constexpr (A::kExact) ur = uvs[RLT2_IDX(r, m > 0 ? m : 1)];
-      else ur = __shfl_sync(kFull, u, gb + r);
+      const double ur = __shfl_sync(kFull, u, gb + r);
       if (relaxing && !scanned) {
-        const T nd = A::add(dm, A::sub(A::sub(cs[RLT2_IDX(r, m) * ld + gl], ur), v));
-        if (A::kExact ? nd < d : A::key(nd) < dk) {
+        const double nd = dadd(dm, dsub(dsub(cs[RLT2_IDX(r, m) * ld + gl], ur), v));
+        if (okey(nd) < dk) {
           d = nd;
-          if constexpr (!A::kExact) dk = A::key(nd);
+          dk = okey(nd);
           pred = r;
         }
       }
@@ -403,7 +300,7 @@ __device__ __forceinline__ WarpLapResult<typename A::T> group_lap(typename A::T*
     // m - k columns still unscanned
     const int step = __popc(group_bits<G>(__ballot_sync(kFull, act && cv && scanned), gb)) - 1;
     if (act) nrelax += step * m - (step * (step + 1)) / 2;
-    if (act && cv && scanned) v = A::add(v, A::sub(d, dlast));
+    if (act && cv && scanned) v = dadd(v, dsub(d, dlast));
     // augment back to row i (groups walk their own chains in lockstep)
     bool walking = act;
     int col = sink;
@@ -418,52 +315,28 @@ __device__ __forceinline__ WarpLapResult<typename A::T> group_lap(typename A::T*
       }
     }
     const int mc = (cv && r2c >= 0) ? r2c : 0;
-    const T vm = __shfl_sync(kFull, v, gb + mc);
-    if (act && cv && r2c >= 0) u = A::sub(cs[gl * ld + RLT2_IDX(r2c, m)], vm);
-    if constexpr (A::kExact) {
-      uvs[gl] = u;
-      __syncwarp();
-    }
+    const double vm = __shfl_sync(kFull, v, gb + mc);
+    if (act && cv && r2c >= 0) u = dsub(cs[gl * ld + RLT2_IDX(r2c, m)], vm);
   }
 
   // optimum: pairwise tree over P = next power of two >= m rows (empty rows add
   // nothing), lane i adding lane i + h for h = P/2, ..., 1
-  const T xr = cv ? cs[gl * ld + RLT2_IDX(r2c, m)] : T(0);
-  T val;
-  if constexpr (G == 32 && A::kExact) {
-    // exact sums do not depend on the order: the 64-bit entries as two
-    // non-negative 26-bit limbs and a signed top part, each summed over the
-    // warp by one 32-bit reduction (32 limbs < 2^31, no overflow)
-    const unsigned long long ux = (unsigned long long)xr;
-    const int l0 = (int)(ux & 0x3ffffffull), l1 = (int)((ux >> 26) & 0x3ffffffull);
-    const int l2 = (int)(xr >> 52);
-    const long long s0 = __reduce_add_sync(kFull, l0), s1 = __reduce_add_sync(kFull, l1);
-    const long long s2 = __reduce_add_sync(kFull, l2);
-    val = (T)(s2 * (1ll << 52) + s1 * (1ll << 26) + s0);
-  } else {
-    int P = 1;
-    while (P < m) P <<= 1;
-    const int PM = (G == 32) ? P : (int)__reduce_max_sync(kFull, (unsigned)P);
-    val = xr;
-    for (int h = PM >> 1; h >= 1; h >>= 1) {
-      const T o = __shfl_xor_sync(kFull, val, h);
-      if (h < P) val = A::add(val, o);
-    }
-    val = __shfl_sync(kFull, val, gb);
+  const double xr = cv ? cs[gl * ld + RLT2_IDX(r2c, m)] : 0.0;
+  int P = 1;
+  while (P < m) P <<= 1;
+  const int PM = (G == 32) ? P : (int)__reduce_max_sync(kFull, (unsigned)P);
+  double val = xr;
+  for (int h = PM >> 1; h >= 1; h >>= 1) {
+    const double o = __shfl_xor_sync(kFull, val, h);
+    if (h < P) val = dadd(val, o);
   }
+  val = __shfl_sync(kFull, val, gb);
 
   if (dual_mode != 0) {
     // canonical duals: shortest paths from row 0 on reduced weights
     // pi(r, sigma(r')) = (c_{r,sigma(r')} - u_r) - v_{sigma(r')} >= 0
     const int s0 = __shfl_sync(kFull, r2c, gb);
-    // exact form: a lane forms only the reduced costs of its own row that the
-    // pass reads (two integer subtractions each, with the column duals
-    // broadcast from shared memory) instead of the whole reduced tile first
-    constexpr bool kRed = PRE && !A::kExact;  // the reduced tile is formed first
-    if constexpr (A::kExact) {
-      uvs[32 + gl] = v;
-      __syncwarp();
-    } else if constexpr (PRE) {
+    if constexpr (PRE) {
       // an FP64 instruction costs the same with few lanes active, so the group's
       // lanes take the m*m entries in row-major turns (every lane busy); (r, c)
       // of entry gl + k*G advance without a division per entry
@@ -474,7 +347,7 @@ __device__ __forceinline__ WarpLapResult<typename A::T> group_lap(typename A::T*
         const int qg = G / m, rg = G - qg * m;
         int r = gl / m, c = gl - r * m;
         for (; r < m; r += qg) {
-          cs[r * ld + c] = A::sub(A::sub(cs[r * ld + c], uvs[r]), uvs[32 + c]);
+          cs[r * ld + c] = dsub(dsub(cs[r * ld + c], uvs[r]), uvs[32 + c]);
           c += rg;
           if (c >= m) {
             c -= m;
@@ -484,48 +357,322 @@ __device__ __forceinline__ WarpLapResult<typename A::T> group_lap(typename A::T*
       }
       __syncwarp();
     }
-    T vs0 = T(0);
-    if constexpr (A::kExact) vs0 = uvs[32 + RLT2_IDX(s0 < 0 ? 0 : s0, m > 0 ? m : 1)];
-    else vs0 = __shfl_sync(kFull, v, gb + (s0 < 0 ? 0 : s0));
-    T dist = T(0);
+    const double vs0 = __shfl_sync(kFull, v, gb + (s0 < 0 ? 0 : s0));
+    double dist = 0.0;
     if (cv && gl != 0) {
-      if constexpr (kRed) dist = cs[gl * ld + RLT2_IDX(s0, m)];
-      else dist = A::sub(A::sub(cs[gl * ld + RLT2_IDX(s0, m)], u), vs0);
+      if constexpr (PRE) dist = cs[gl * ld + RLT2_IDX(s0, m)];
+      else dist = dsub(dsub(cs[gl * ld + RLT2_IDX(s0, m)], u), vs0);
     }
     bool done = !cv || gl == 0;
-    unsigned long long dk = A::key(dist);  // cached key of dist (rounded form only)
+    unsigned long long dk = okey(dist);  // cached key of dist
     for (int it = 0; it < M - 2; ++it) {
       const bool stepping = it < m - 2;
-      const int rs = group_argmin<G>(done ? ~0ull : (A::kExact ? A::key(dist) : dk), gb);
-      const T dr = __shfl_sync(kFull, dist, gb + rs);
+      const int rs = group_argmin<G>(done ? ~0ull : dk, gb);
+      const double dr = __shfl_sync(kFull, dist, gb + rs);
       if (stepping && gl == rs) done = true;
       const int s = __shfl_sync(kFull, r2c, gb + rs);
-      T vs = T(0);
-      if constexpr (A::kExact) vs = uvs[32 + RLT2_IDX(s < 0 ? 0 : s, m > 0 ? m : 1)];
-      else if constexpr (!kRed) vs = __shfl_sync(kFull, v, gb + (s < 0 ? 0 : s));
+      double vs = 0.0;
+      if constexpr (!PRE) vs = __shfl_sync(kFull, v, gb + (s < 0 ? 0 : s));
       if (stepping && !done) {
-        T w;
-        if constexpr (kRed) w = cs[gl * ld + RLT2_IDX(s, m)];
-        else w = A::sub(A::sub(cs[gl * ld + RLT2_IDX(s, m)], u), vs);
-        const T nd = A::add(dr, w);
-        if (A::kExact ? nd < dist : A::key(nd) < dk) {
+        double w;
+        if constexpr (PRE) w = cs[gl * ld + RLT2_IDX(s, m)];
+        else w = dsub(dsub(cs[gl * ld + RLT2_IDX(s, m)], u), vs);
+        const double nd = dadd(dr, w);
+        if (okey(nd) < dk) {
           dist = nd;
-          if constexpr (!A::kExact) dk = A::key(nd);
+          dk = okey(nd);
         }
       }
     }
-    const T u0r = __shfl_sync(kFull, u, gb);
-    const T ucan = cv ? (m > 1 ? A::add(dist, A::sub(u, u0r)) : T(0)) : T(0);
+    const double u0r = __shfl_sync(kFull, u, gb);
+    const double ucan = cv ? (m > 1 ? dadd(dist, dsub(u, u0r)) : 0.0) : 0.0;
     // v_c = c_{sigma^-1(c), c} - u_{sigma^-1(c)}, from the matched row's own entry
-    const T wrow = A::sub(xr, ucan);
+    const double wrow = dsub(xr, ucan);
     const int rr = cv ? c2r : 0;
-    const T vcan = __shfl_sync(kFull, wrow, gb + rr);
+    const double vcan = __shfl_sync(kFull, wrow, gb + rr);
     u = ucan;
-    v = cv ? vcan : T(0);
-    if constexpr (A::kExact) __syncwarp();  // the reads of uvs are done before a caller reuses it
+    v = cv ? vcan : 0.0;
   }
   R.u = u;
   R.v = v;
+  R.r2c = r2c;
+  R.c2r = c2r;
+  R.value = val;
+  R.naug = naug;
+  R.nrelax = nrelax;
+  return R;
+}
+
+// ---- exact form --------------------------------------------------------------
+// Group lane of the least (kh, lo) pair, lowest lane on ties; a lane out of the
+// race holds kh = ~0 (labels and distances are in [0, 2^58), so the high word of
+// one in the race is smaller).  The low words are compared only where several
+// lanes of a group share the least high word.  Every lane of the warp calls it.
+template <int G>
+__device__ __forceinline__ int fx_argmin(unsigned kh, unsigned lo, int gb) {
+  if constexpr (G == 32) {
+    const unsigned mh = __reduce_min_sync(kFull, kh);
+    unsigned ball = __ballot_sync(kFull, kh == mh);
+    if (ball & (ball - 1u)) {
+      const unsigned ml = __reduce_min_sync(kFull, kh == mh ? lo : 0xffffffffu);
+      ball = __ballot_sync(kFull, kh == mh && lo == ml);
+    }
+    return __ffs(ball) - 1;
+  } else {
+    constexpr unsigned mask = (1u << G) - 1u;
+    auto group_min = [&](unsigned x) {
+      if constexpr (G == 16) {
+        // two full-warp reductions, each with the other half at the maximum (no
+        // divergence, unlike a redux.sync on a half-warp mask)
+        const unsigned a = __reduce_min_sync(kFull, gb ? 0xffffffffu : x);
+        const unsigned b = __reduce_min_sync(kFull, gb ? x : 0xffffffffu);
+        return gb ? b : a;
+      } else {
+#pragma unroll
+        for (int off = G / 2; off > 0; off >>= 1) x = min(x, __shfl_xor_sync(kFull, x, off));
+        return x;
+      }
+    };
+    const unsigned mh = group_min(kh);
+    unsigned mine = (__ballot_sync(kFull, kh == mh) >> gb) & mask;
+    if (__any_sync(kFull, (mine & (mine - 1u)) != 0u)) {
+      const unsigned ml = group_min(kh == mh ? lo : 0xffffffffu);
+      mine = (__ballot_sync(kFull, kh == mh && lo == ml) >> gb) & mask;
+    }
+    return __ffs(mine) - 1;
+  }
+}
+
+// fx_floor_entry from the entry's words, kk = (L + 1075) << 20: sign, hidden bit
+// (0 for exponent field 0) and shift without a branch.
+__device__ __forceinline__ long long fx_floor_words(unsigned hi, unsigned lo, unsigned kk) {
+  const unsigned ex = hi & 0x7ff00000u;
+  const unsigned long long mant = ((unsigned long long)((hi & 0xfffffu) | min(ex, 0x100000u)) << 32) | lo;
+  const long long neg = (long long)((int)hi >> 31);
+  long long q;
+  // 64-bit shifts by 64 and more leave the sign
+  asm("shr.s64 %0, %1, %2;" : "=l"(q) : "l"(((long long)mant ^ neg) - neg), "r"((kk - max(ex, 0x100000u)) >> 20));
+  return q;
+}
+
+// One LAP per group of G lanes in exact fixed point with canonical duals: the
+// algorithm, tie rules and hence the results (assignment and counters too) are
+// those of group_lap; exact sums may be taken in any order, so a step costs
+// fewer instructions:
+//   - column lane c keeps um = u of its matched row, and row duals exist in
+//     shared memory only for free rows (uvs, the start duals): a step's
+//     broadcast is d_c - um_c in one shuffle pair, its relaxation
+//     (c_rc - v_c) + that, and the dual update touches the column lane alone
+//     (a matched edge stays tight, so u falls by what v rises);
+//   - the predecessor of a column is the column scanned before it, so the
+//     augmenting path is a mask of columns and all its columns take their
+//     new rows at once;
+//   - lanes out of the race are marked in the word that the argmin compares;
+//   - at one LAP per warp every loop condition is warp-uniform and needs no vote.
+// raw (nullable): the tile as doubles with row stride rs, in shared memory and
+// possibly the tile itself; the column reduction converts it into cs and then
+// calls hook().  kk = (L + 1075) << 20 for the tile's grid 2^L.
+// Bound by the ALU pipe (77 % busy) and issue (80 %).  Z stage, warm: n = 20 394
+// -> 370 us (3,160 -> 2,840 warp instructions per LAP: 580 the column
+// reduction, 950 the searches, 650 the canonical pass), n = 17 160 -> 139,
+// n = 12 41.5 -> 34.
+template <int G, bool RR = false, typename Hook = NoHook>
+__device__ __forceinline__ WarpLapResult<long long> group_lap_fx(long long* cs, int ld, int m, int lane, bool warm,
+                                                                 long long u0, int* scr, long long* uvs,
+                                                                 const double* raw = nullptr, int rs = 0, int L = 0,
+                                                                 const Hook& hook = Hook()) {
+  using T = long long;
+  constexpr unsigned kOut = 0xffffffffu;
+  constexpr T kTop = 0x7fffffffffffffffll;
+  const int gl = lane & (G - 1), gb = lane - gl;
+  const bool cv = gl < m;
+  const int gc = cv ? gl : 0;  // a lane past the LAP reads column 0
+  const int M = (G == 32) ? m : (int)__reduce_max_sync(kFull, (unsigned)m);
+  auto hi32 = [](T x) { return (unsigned)((unsigned long long)x >> 32); };
+  const unsigned kk = (unsigned)(L + 1075) << 20;
+  auto entry = [&](int r) {  // column gl's entry of row r, onto the grid
+    const uint2 w = *reinterpret_cast<const uint2*>(raw + r * rs + gl);
+    const T c = fx_floor_words(w.y, w.x, kk);
+    cs[r * ld + gl] = c;
+    return c;
+  };
+  T u = (cv && warm) ? u0 : T(0);
+  if constexpr (RR) {
+    if (!__any_sync(kFull, warm)) {  // warp-uniform: the launches with RR start every LAP cold
+      if (raw) {
+        if (cv)
+          for (int r = 0; r < m; ++r) entry(r);
+        __syncwarp();
+        hook();
+        raw = nullptr;
+      }
+      T mn = kTop;
+      if (cv)
+        for (int c = 0; c < m; ++c) {  // lane = row (odd row stride: no bank conflicts)
+          const T x = cs[gl * ld + c];
+          mn = x < mn ? x : mn;
+        }
+      u = cv ? mn : T(0);
+    }
+  }
+  uvs[gl] = u;
+  __syncwarp();
+  // column reduction with the argmin row
+  T v = kTop;
+  int arg = 0;
+  if (cv) {
+    auto reduce = [&](int r, T c) {
+      const T x = c - uvs[r];
+      if (x < v) {
+        v = x;
+        arg = r;
+      }
+    };
+    if (raw) {
+#pragma unroll 3
+      for (int r = 0; r < m; ++r) reduce(r, entry(r));
+    } else {
+#pragma unroll 3
+      for (int r = 0; r < m; ++r) reduce(r, cs[r * ld + gl]);
+    }
+  } else {
+    v = T(0);
+  }
+  if (raw) {
+    __syncwarp();  // every lane's reads of raw are done
+    hook();
+  }
+  // greedy: the lowest column among those sharing an argmin row takes it
+  const unsigned same = __match_any_sync(kFull, cv ? (gb << 6) + arg : (1 << 20) + lane);
+  const bool win = cv && (__ffs(same) - 1) == lane;
+  int c2r = win ? arg : -1;
+  T um = uvs[arg];  // used where the column is matched
+  unsigned taken = __reduce_or_sync(kFull, win ? 1u << (gb + arg) : 0u);
+  unsigned freerows = (m > 0 ? kFull >> (32 - m) : 0u) & ~(taken >> gb);
+  int naug = 0, nrelax = 0;
+  while (G == 32 ? freerows != 0 : __any_sync(kFull, freerows != 0)) {
+    const bool act = freerows != 0;  // this group runs a search in this pass
+    const int i = act ? __ffs(freerows) - 1 : 0;
+    if (act) {
+      freerows &= freerows - 1;
+      ++naug;
+      nrelax += m;
+    }
+    T d = (cs[i * ld + gc] - uvs[i]) - v;
+    unsigned kh = (act && cv) ? hi32(d) : kOut;
+    int from = -1;  // the column scanned before this one on its path (-1: reached from row i)
+    int sink = 0;
+    bool searching = act;
+    // the free columns as a mask: at one LAP per warp the test is then on
+    // uniform values
+    const unsigned freecols = __ballot_sync(kFull, cv && c2r < 0) >> gb;
+    while (G == 32 ? true : __any_sync(kFull, searching)) {
+      const int c = fx_argmin<G>(kh, (unsigned)d, gb);
+      if (G == 32 || searching) {
+        if ((freecols >> c) & 1u) {
+          sink = c;
+          if constexpr (G == 32) break;
+          searching = false;
+        }
+      }
+      const int r0 = __shfl_sync(kFull, c2r, gb + c);
+      const T es = __shfl_sync(kFull, d - um, gb + c);
+      if (G == 32 || searching) {
+        if (gl == c) kh = kOut;
+        const T nd = (cs[RLT2_IDX(r0, m) * ld + gc] - v) + es;
+        if (kh != kOut && nd < d) {
+          d = nd;
+          kh = hi32(nd);
+          from = c;
+        }
+      }
+    }
+    // the k-th scanned column relaxed the m - k columns still unscanned
+    const bool scanned = act && cv && kh == kOut;
+    const int step = __popc(group_bits<G>(__ballot_sync(kFull, scanned), gb));
+    if (act) nrelax += step * m - (step * (step + 1)) / 2;
+    const T dlast = __shfl_sync(kFull, d, gb + sink);
+    if (scanned) {
+      const T delta = d - dlast;
+      v += delta;
+      um -= delta;
+    }
+    // the path's columns, then their new rows at once
+    const int row = __shfl_sync(kFull, c2r, gb + (from < 0 ? 0 : from));
+    unsigned path = 0;
+    int col = sink;
+    bool walking = act;
+    while (G == 32 ? true : __any_sync(kFull, walking)) {
+      if (walking) path |= 1u << col;
+      if constexpr (G == 32) {
+        const int p = (int)__reduce_max_sync(kFull, lane == col ? (unsigned)(from + 1) : 0u);
+        if (p == 0) break;
+        col = p - 1;
+      } else {
+        const int p = __shfl_sync(kFull, from, gb + col);
+        walking = walking && p >= 0;
+        if (walking) col = p;
+      }
+    }
+    if ((path >> gl) & 1u) {
+      c2r = from < 0 ? i : row;
+      um = cs[RLT2_IDX(c2r, m) * ld + gc] - v;
+    }
+  }
+  // to row lanes: the matched column and the row dual
+  __syncwarp();
+  if (cv) {
+    scr[c2r] = gl;
+    uvs[c2r] = um;
+  }
+  __syncwarp();
+  const int r2c = cv ? scr[gl] : 0;
+  u = cv ? uvs[gl] : T(0);
+  const T vown = __shfl_sync(kFull, v, gb + r2c);  // dual of the matched column
+  const T xr = cv ? u + vown : T(0);               // the assigned entry
+  T val;
+  if constexpr (G == 32) {
+    // the 64-bit entries as two non-negative 26-bit limbs and a signed top
+    // part, each summed over the warp by one 32-bit reduction (no overflow)
+    const unsigned long long ux = (unsigned long long)xr;
+    const long long s0 = __reduce_add_sync(kFull, (int)(ux & 0x3ffffffull));
+    const long long s1 = __reduce_add_sync(kFull, (int)((ux >> 26) & 0x3ffffffull));
+    const long long s2 = __reduce_add_sync(kFull, (int)(xr >> 52));
+    val = s2 * (1ll << 52) + s1 * (1ll << 26) + s0;
+  } else {
+    val = xr;
+#pragma unroll
+    for (int h = G / 2; h >= 1; h >>= 1) val += __shfl_xor_sync(kFull, val, h);
+  }
+  // canonical duals: Dijkstra from row 0 over arcs r' -> r of weight
+  // (c_{r,sigma(r')} - u_r) - v_{sigma(r')}; row lanes broadcast dist - v_own
+  T dist = 1ll << 61;  // above every distance
+  unsigned kh = cv ? hi32(dist) : kOut;
+  if (gl == 0) {
+    dist = T(0);
+    kh = kOut;
+  }
+  int rs0 = 0;
+  for (int it = 0; it < M - 1; ++it) {
+    const T es = __shfl_sync(kFull, dist - vown, gb + rs0);
+    const int s = __shfl_sync(kFull, r2c, gb + rs0);
+    if (G == 32 || it < m - 1) {
+      if (gl == rs0) kh = kOut;
+      const T nd = (cs[gc * ld + RLT2_IDX(s, m > 0 ? m : 1)] - u) + es;
+      if (kh != kOut && nd < dist) {
+        dist = nd;
+        kh = hi32(nd);
+      }
+    }
+    if (it + 2 < M) rs0 = fx_argmin<G>(kh, (unsigned)dist, gb);
+  }
+  const T u0r = __shfl_sync(kFull, u, gb);
+  const T ucan = cv ? dist + (u - u0r) : T(0);
+  const T vcan = __shfl_sync(kFull, xr - ucan, gb + (cv ? c2r : 0));
+  __syncwarp();  // the reads of uvs and scr are done before a caller reuses them
+  WarpLapResult<T> R;
+  R.u = ucan;
+  R.v = cv ? vcan : T(0);
   R.r2c = r2c;
   R.c2r = c2r;
   R.value = val;
@@ -548,6 +695,11 @@ __host__ __device__ inline size_t warp_smem_bytes(int m, int G) {
 __host__ __device__ inline size_t raw_group_doubles(int m) { return ((size_t)m * m + m + 1) & ~size_t(1); }
 __host__ __device__ inline size_t warp_smem_bytes_async(int m, int G) {
   return warp_smem_bytes(m, G) + (size_t)(32 / G) * raw_group_doubles(m) * sizeof(double);
+}
+
+// The one-tile form (G = 32): the tile, 32 dual slots and 32 ints.
+__host__ __device__ inline size_t warp_smem_bytes_one(int m) {
+  return (size_t)m * tile_ld(m) * sizeof(double) + 32 * sizeof(double) + 32 * sizeof(int);
 }
 
 // Stages one group's tile (plus an optional addend) into shared memory, the
@@ -612,6 +764,10 @@ __device__ __forceinline__ int stage_tile(typename std::conditional<FX, long lon
     return L;
   }
 }
+
+// Reduced costs: rounded in FP64, exact on the grid.
+__device__ __forceinline__ double lap_sub(double a, double b) { return __dsub_rn(a, b); }
+__device__ __forceinline__ long long lap_sub(long long a, long long b) { return a - b; }
 
 template <bool FX, typename T>
 __device__ __forceinline__ double out_value(T x, int L) {
