@@ -150,6 +150,9 @@ int default_group(int m);
 // outside stream capture before the first launch of that size.
 cudaError_t prepare_lap(int m, int group = 0, int warps_per_block = 0);
 
+// The same for the three LAP stages of an n-facility iteration (ascent.cu).
+cudaError_t prepare_lap_stages(int n);
+
 // Enqueue the batched LAP kernel (grid sized for the device); returns the CUDA error.
 cudaError_t launch_lap(const LapArgs& a, cudaStream_t s);
 
