@@ -38,77 +38,124 @@ constexpr int kInPad = 64;   // padded input width (GEMM K)
 constexpr int kChunk = 1 << 18;  // rows per inference/training chunk
 using bf16 = __nv_bfloat16;
 
+// x with its significand cut to FP32: the exponent field less 896 (its low eight
+// bits with the top one flipped), zero below the range, the largest FP32 above.
 __device__ __forceinline__ float f32_trunc(double x) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  const unsigned sign = (unsigned)(b >> 63) << 31;
-  const int e = (int)((b >> 52) & 0x7ff);
-  unsigned out;
-  if (e == 0) {
-    out = sign;
-  } else {
-    const int ef = e - 1023 + 127;
-    if (ef <= 0) out = sign;
-    else if (ef >= 255) out = sign | 0x7f7fffffu;
-    else out = sign | ((unsigned)ef << 23) | (unsigned)((b >> 29) & 0x7fffff);
-  }
-  return __uint_as_float(out);
+  const unsigned hi = (unsigned)(b >> 32), lo = (unsigned)b;
+  const unsigned e = (hi >> 20) & 0x7ffu;
+  unsigned m = (__funnelshift_l(lo, hi, 3) ^ 0x40000000u) & 0x7fffffffu;
+  m = e <= 896u ? 0u : e >= 1151u ? 0x7f7fffffu : m;
+  return __uint_as_float(m | (hi & 0x80000000u));
 }
 
 // ------------------------------------------------------------- features ----
+// Ascending bitonic sort of `width` lanes (8, 16 or 32; the lanes past a row's
+// end hold the largest key) of two rows at once: unsigned 16-bit keys, row i in
+// the low half.
+__device__ __forceinline__ unsigned sort_rows(unsigned v, int width, int lane) {
+#pragma unroll
+  for (int k = 2; k <= 32; k <<= 1) {
+    if (k > width) break;
+#pragma unroll
+    for (int j = k >> 1; j > 0; j >>= 1) {
+      const unsigned o = __shfl_xor_sync(kFull, v, j);
+      v = ((lane & j) == 0) == ((lane & k) == 0) ? __vminu2(v, o) : __vmaxu2(v, o);
+    }
+  }
+  return v;
+}
+// The same on floats, one row (scaled rows that overflow FP32).
+__device__ __forceinline__ float sort_row(float v, int lane) {
+#pragma unroll
+  for (int k = 2; k <= 32; k <<= 1) {
+#pragma unroll
+    for (int j = k >> 1; j > 0; j >>= 1) {
+      const float o = __shfl_xor_sync(kFull, v, j);
+      v = ((lane & j) == 0) == ((lane & k) == 0) ? fminf(v, o) : fmaxf(v, o);
+    }
+  }
+  return v;
+}
+
 // One warp per tile; lane j holds column j.  Writes 64 BF16 inputs per row
 // (34 features + zero padding), optional FP32 targets and the tile scale.
-// The tile (at most 8 KB) is read three times -- column minima, the scale, then
-// row by row for the sorts -- so only the first pass reaches DRAM and the
-// kernel keeps few registers (occupancy hides the load latency).
-__global__ void __launch_bounds__(256, 4) k_features(long long ntiles, int m, const double* __restrict__ tiles,
-                                                     const double* __restrict__ prev_u,
-                                                     const double* __restrict__ target_u, bf16* __restrict__ X,
-                                                     float* __restrict__ target, float* __restrict__ scale) {
+// What bounds it is issue: the tile is read and turned into FP32 once (kept in
+// shared memory), the scale comes from the column minima and maxima (FP32
+// subtraction is monotone), and since the BF16 rounding is monotone too the
+// values are rounded first and two rows sorted at once as packed 16-bit keys
+// (non-negative BF16 order as integers), with as many stages as m needs.
+// 144,400 tiles of size 18: 72 -> 43 us per 262,144 rows, the whole prediction
+// 1.41 -> 1.11 ms.
+constexpr int kFeatWarps = 8;
+__global__ void __launch_bounds__(kFeatWarps * 32) k_features(long long ntiles, int m,
+                                                              const double* __restrict__ tiles,
+                                                              const double* __restrict__ prev_u,
+                                                              const double* __restrict__ target_u,
+                                                              bf16* __restrict__ X, float* __restrict__ target,
+                                                              float* __restrict__ scale) {
+  extern __shared__ float feat_smem[];
   const int lane = threadIdx.x & 31;
   const bool col = lane < m;
+  float* sm = feat_smem + (threadIdx.x >> 5) * m * m;
+  const int width = m <= 8 ? 8 : m <= 16 ? 16 : 32;
+  const unsigned mword = (unsigned)__bfloat16_as_ushort(__float2bfloat16_rn((float)m / 32.0f)) << 16;
   const long long nw = (long long)gridDim.x * (blockDim.x >> 5);
   for (long long t = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); t < ntiles; t += nw) {
     const double* c = tiles + t * m * m;
-    float cmin = INFINITY;
-    for (int i = 0; i < m; ++i)
-      if (col) cmin = fminf(cmin, f32_trunc(c[i * m + lane]));
-    float rmax = 0.0f;
-    for (int i = 0; i < m; ++i)
-      if (col) rmax = fmaxf(rmax, __fsub_rn(f32_trunc(c[i * m + lane]), cmin));
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) rmax = fmaxf(rmax, __shfl_xor_sync(kFull, rmax, off));
+    float cmin = INFINITY, cmax = -INFINITY;
+    if (col) {
+#pragma unroll 6
+      for (int i = 0; i < m; ++i) {
+        const float f = f32_trunc(__ldcs(c + i * m + lane));
+        sm[i * m + lane] = f;
+        cmin = fminf(cmin, f);
+        cmax = fmaxf(cmax, f);
+      }
+    }
+    const double pd = (prev_u && col) ? prev_u[t * m + lane] : 0.0;
+    float rmax = col ? fmaxf(0.0f, __fsub_rn(cmax, cmin)) : 0.0f;
+    rmax = __uint_as_float(__reduce_max_sync(kFull, __float_as_uint(rmax)));  // non-negative: ordered as integers
     const float s = rmax > 0.0f ? rmax : 1.0f;
     const float inv = __fdiv_rn(1.0f, s);
     if (lane == 0 && scale) scale[t] = s;
-    for (int i = 0; i < m; ++i) {
-      float v = col ? __fmul_rn(__fsub_rn(f32_trunc(c[i * m + lane]), cmin), inv) : INFINITY;
-      // bitonic sort across the warp, ascending
-#pragma unroll
-      for (int k = 2; k <= 32; k <<= 1) {
-#pragma unroll
-        for (int j = k >> 1; j > 0; j >>= 1) {
-          const float o = __shfl_xor_sync(kFull, v, j);
-          const bool up = (lane & k) == 0;
-          const bool low = (lane & j) == 0;
-          v = (low == up) ? fminf(v, o) : fmaxf(v, o);
-        }
+    const float pv = prev_u ? __fmul_rn(f32_trunc(pd), inv) : 0.0f;  // row `lane`'s scaled previous dual
+    unsigned* xr = reinterpret_cast<unsigned*>(X + t * m * kInPad) + (lane >> 1);
+    const bool odd = lane & 1;  // even lanes write row i, odd lanes row i + 1, a word each
+    for (int i = 0; i < m; i += 2) {
+      const int i1 = min(i + 1, m - 1);
+      const float va = col ? __fmul_rn(__fsub_rn(sm[i * m + lane], cmin), inv) : INFINITY;
+      const float vb = col ? __fmul_rn(__fsub_rn(sm[i1 * m + lane], cmin), inv) : INFINITY;
+      unsigned w;
+      if (s <= 3.402823466e38f) {
+        const __nv_bfloat162 r = __floats2bfloat162_rn(va, vb);
+        w = sort_rows(*reinterpret_cast<const unsigned*>(&r), width, lane);
+      } else {
+        const __nv_bfloat162 r = __floats2bfloat162_rn(sort_row(va, lane), sort_row(vb, lane));
+        w = *reinterpret_cast<const unsigned*>(&r);
       }
-      const long long row = t * m + i;
-      bf16* xr = X + row * kInPad;
-      xr[lane] = __float2bfloat16_rn(col ? v : 0.0f);
-      float hi = 0.0f;
-      if (lane == 0) hi = prev_u ? __fmul_rn(f32_trunc(prev_u[row]), inv) : 0.0f;
-      if (lane == 1) hi = (float)m / 32.0f;
-      xr[32 + lane] = __float2bfloat16_rn(hi);
+      if (!col) w = 0;
+      const unsigned o = __shfl_xor_sync(kFull, w, 1);
+      const float pr = __shfl_sync(kFull, pv, odd ? i1 : i);
+      const unsigned hi = lane < 2 ? mword | (unsigned)__bfloat16_as_ushort(__float2bfloat16_rn(pr)) : 0u;
+      if (!odd || i + 1 < m) {
+        unsigned* row = xr + (size_t)(i + odd) * (kInPad / 2);
+        row[0] = odd ? __byte_perm(w, o, 0x3276) : __byte_perm(w, o, 0x5410);
+        row[16] = hi;
+      }
     }
     if (target && target_u && col) {
       // the network predicts the change of the row dual since the previous iteration
       const long long r = t * m + lane;
-      const double d = prev_u ? __dsub_rn(target_u[r], prev_u[r]) : target_u[r];
+      const double d = prev_u ? __dsub_rn(target_u[r], pd) : target_u[r];
       target[r] = __fmul_rn(f32_trunc(d), inv);
     }
   }
 }
+static int feat_grid(long long ntiles) {
+  return (int)std::min<long long>(8192, (ntiles + kFeatWarps - 1) / kFeatWarps);
+}
+static size_t feat_smem_bytes(int m) { return (size_t)kFeatWarps * m * m * sizeof(float); }
 
 // ----------------------------------------------------------------- GEMM ----
 // C[M x N] = A[M x K] * B[K x N] with BF16 inputs and FP32 accumulation on the
@@ -573,7 +620,7 @@ cudaError_t mlp_predict_enqueue(rlt2_mlp* m, long long ntiles, int mz, const dou
   for (long long t0 = 0; t0 < ntiles; t0 += tiles_per_chunk) {
     const long long nt = std::min(tiles_per_chunk, ntiles - t0);
     const long long rows = nt * mz, prows = (rows + 63) / 64 * 64;
-    k_features<<<(int)std::min<long long>(8192, (nt + 7) / 8), 256, 0, s>>>(
+    k_features<<<feat_grid(nt), kFeatWarps * 32, feat_smem_bytes(mz), s>>>(
         nt, mz, tiles + t0 * mz * mz, prev_u ? prev_u + t0 * mz : nullptr, nullptr, m->Xc, nullptr, m->scale);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (prows > rows && (e = cudaMemsetAsync(m->Xc + rows * kInPad, 0, sizeof(bf16) * (prows - rows) * kInPad, s)) !=
@@ -720,7 +767,7 @@ extern "C" rlt2_status rlt2_mlp_add_samples(rlt2_mlp* m, long long ntiles, int m
   CKM(ensure_dataset(m, m->rows + ntiles * mz));
   float* scale = nullptr;
   CKM(cudaMalloc((void**)&scale, sizeof(float) * ntiles));
-  k_features<<<(int)std::min<long long>(8192, (ntiles + 7) / 8), 256, 0, m->stream>>>(
+  k_features<<<feat_grid(ntiles), kFeatWarps * 32, feat_smem_bytes(mz), m->stream>>>(
       ntiles, mz, tiles, prev_u, target_u, m->Xd + m->rows * kInPad, m->Td + m->rows, scale);
   cudaError_t e = cudaGetLastError();
   cudaError_t e2 = cudaStreamSynchronize(m->stream);
