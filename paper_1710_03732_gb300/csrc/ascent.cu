@@ -614,14 +614,6 @@ static rlt2_status ctx_alloc(rlt2_ctx* c, bool own_qap) {
   return RLT2_OK;
 }
 
-// The launches of enqueue_iteration's three LAP stages (outside stream capture).
-cudaError_t rlt2::prepare_lap_stages(int n) {
-  cudaError_t e = prepare_lap(n - 2);
-  if (e == cudaSuccess) e = prepare_lap(n - 1, 32, 4);
-  if (e == cudaSuccess) e = prepare_lap(n, 32);
-  return e;
-}
-
 extern "C" rlt2_status rlt2_create(int n, const double* F, const double* D, const double* B, const int* partial,
                                    const rlt2_params* p, void* stream, rlt2_ctx** out) {
   if (!out) {
@@ -735,7 +727,7 @@ extern "C" rlt2_status rlt2_create(int n, const double* F, const double* D, cons
   if (e != cudaSuccess) return fail(e, "setup kernels");
   if (e3 != cudaSuccess) return fail(e3, "setup sync");
   if ((e = cudaMemcpy(&c->cst_host, c->d_cst, 8, cudaMemcpyDeviceToHost)) != cudaSuccess) return fail(e, "cst");
-  if ((e = prepare_lap_stages(nr)) != cudaSuccess) return fail(e, "prepare_lap");
+  if ((e = prepare_lap(nr - 2)) != cudaSuccess) return fail(e, "prepare_lap");
   *out = c;
   return RLT2_OK;
 }
@@ -808,7 +800,7 @@ extern "C" rlt2_status rlt2_create_child(rlt2_ctx* parent, int facility, int loc
   if (e == cudaSuccess) e = cudaMemcpyAsync(&c->sc->lb_base, c->d_cst, sizeof(double), cudaMemcpyDeviceToDevice, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e == cudaSuccess) e = cudaMemcpy(&c->cst_host, c->d_cst, 8, cudaMemcpyDeviceToHost);
-  if (e == cudaSuccess) e = prepare_lap_stages(nr);
+  if (e == cudaSuccess) e = prepare_lap(nr - 2);
   if (e != cudaSuccess) {
     rlt2_status r = cuda_fail(e, "rlt2_create_child");
     ctx_free(c);
@@ -1025,12 +1017,8 @@ cudaError_t rlt2::enqueue_iteration(const IterView& v, cudaStream_t s, cudaEvent
   y.dual_mode = p.dual_mode;
   y.stats = v.sc->stats + 2;
   y.skip = done;
-  y.warps_per_block = 4;  // n^2 LAPs only: spread them over more SMs
-  // and one LAP per warp at every size: the stage's time is one LAP's latency,
-  // and LAPs that share a warp wait for each other (n = 8: Y 16.7 -> 11.4 us, X 11.7 -> 8.6; n = 17: Y 25.8 -> 18.4)
-  y.group = 32;
   if ((e = rec(3, 0)) != cudaSuccess) return e;
-  if ((e = launch_lap(y, s)) != cudaSuccess) return e;
+  if ((e = launch_lap_blocks(y, s)) != cudaSuccess) return e;
   count(3, 1);
   if ((e = rec(3, 1)) != cudaSuccess) return e;
   // 5) X stage on b' + Delta, writes pi_x
@@ -1049,9 +1037,8 @@ cudaError_t rlt2::enqueue_iteration(const IterView& v, cudaStream_t s, cudaEvent
   x.dual_mode = p.dual_mode;
   x.stats = v.sc->stats + 4;
   x.skip = done;
-  x.group = 32;  // one LAP: no lockstep code
   if ((e = rec(4, 0)) != cudaSuccess) return e;
-  if ((e = launch_lap(x, s)) != cudaSuccess) return e;
+  if ((e = launch_lap_blocks(x, s)) != cudaSuccess) return e;
   count(4, 1);
   if ((e = rec(4, 1)) != cudaSuccess) return e;
   // 6) finalize

@@ -183,122 +183,184 @@ template <int G>
 constexpr int kLapBlocks = G == 16 ? 3 : 4;
 
 // Grid-stride over LAPs, 32/G LAPs per warp per step.  FX selects the exact
-// fixed-point arithmetic (canonical duals), else FP64; RR (fixed point, cold
-// launches) reduces the rows of a cold start first.
-template <int G, bool PRE, bool FX, bool RR = false>
+// fixed-point arithmetic (canonical duals) with prefetching, else FP64; RR
+// (fixed point, cold launches) reduces the rows of a cold start first.
+template <int G, bool FX, bool RR = false>
 __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32, kLapBlocks<G>) k_lap(LapArgs a) {
   if (a.skip && *a.skip) return;
-  using T = typename std::conditional<FX, long long, double>::type;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  if constexpr (FX && PRE) {
-    if (a.prefetch) {
-      const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, wpb = blockDim.x >> 5;
-      const bool warm = a.u0 != nullptr && (a.warm_gate == nullptr || *a.warm_gate != 0);
-      const long long nwarps = (long long)gridDim.x * wpb;
-      if constexpr (G == 32) {
-        if (a.prefetch == 2) {
-          k_lap_one_tile<RR>(a, smem_raw + (size_t)wib * warp_smem_bytes_one(a.m), lane, warm,
-                             (long long)blockIdx.x * wpb + wib, nwarps);
-          return;
-        }
-      }
-      k_lap_prefetching<G, RR>(a, smem_raw + (size_t)wib * warp_smem_bytes_async(a.m, G), lane, warm,
-                           ((long long)blockIdx.x * wpb + wib) * (32 / G), nwarps * (32 / G));
-      return;
-    }
-  }
-  constexpr int per = 32 / G;
-  const int lane = threadIdx.x & 31;
-  const int wib = threadIdx.x >> 5;
-  const int wpb = blockDim.x >> 5;
-  const int grp = lane / G, gl = lane & (G - 1);
-  const int m = a.m;
-  const int ld = tile_ld(m);
-  unsigned char* base = smem_raw + (size_t)wib * warp_smem_bytes(m, G);
-  T* tile = reinterpret_cast<T*>(base) + (size_t)grp * m * ld;
-  T* uv = reinterpret_cast<T*>(base) + (size_t)per * m * ld;  // [0..31] u, [32..63] v
-  int* scr = reinterpret_cast<int*>(uv + 64) + grp * G;
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, wpb = blockDim.x >> 5;
   const bool warm = a.u0 != nullptr && (a.warm_gate == nullptr || *a.warm_gate != 0);
   const long long nwarps = (long long)gridDim.x * wpb;
-  const int mm = m * m;
-  unsigned long long aug_acc = 0, relax_acc = 0;
-
-  for (long long t0 = ((long long)blockIdx.x * wpb + wib) * per; t0 < a.batch; t0 += nwarps * per) {
-    const long long tb = t0 + grp;
-    const bool have = tb < a.batch;
-    const long long t = (have && a.map) ? (long long)a.map[tb] : tb;
-    // with a reduced-cost output (the Y and X stages: few LAPs, one per warp)
-    // the tile's loads are batched
-    const int L = stage_tile<G, FX, false, PRE ? 1 : 4>(tile, ld, m, gl, have ? a.A + t * mm : nullptr,
-                                                        (have && a.Badd) ? a.Badd + t * mm : nullptr);
-    T u0 = T(0);
-    if (warm && have && gl < m) u0 = start_dual<FX>(a.u0[t * m + gl], L);
-    __syncwarp();
-    // without a reduced-cost output (PRE) the tile may be overwritten by the canonical pass
-    WarpLapResult<T> R;
-    if constexpr (FX) R = group_lap_fx<G, RR>(tile, ld, have ? m : 0, lane, warm, u0, scr, uv + grp * G);
-    else R = group_lap<G, PRE>(tile, ld, have ? m : 0, lane, warm, u0, a.dual_mode, scr, uv + grp * G);
-    if (have && gl < m) {
-      if (a.u) a.u[t * m + gl] = out_value<FX>(R.u, L);
-      if (a.v) a.v[t * m + gl] = out_value<FX>(R.v, L);
-      if (a.r2c) a.r2c[t * m + gl] = R.r2c;
-    }
-    if (have && gl == 0) {
-      a.value[t] = out_value<FX>(R.value, L);
-      if (a.naug) a.naug[t] = R.naug;
-      aug_acc += R.naug;
-      relax_acc += R.nrelax;
-    }
-    if (a.pi) {
-      uv[lane] = R.u;
-      uv[32 + lane] = R.v;
-      __syncwarp();
-      if (have) {
-        double* dst = a.pi + t * mm;
-        const T* ug = uv + grp * G;
-        const T* vg = uv + 32 + grp * G;
-#pragma unroll 4
-        for (int e = gl; e < mm; e += G) {
-          const int r = e / m, c = e - r * m;
-          dst[e] = out_value<FX>(lap_sub(lap_sub(tile[r * ld + c], ug[r]), vg[c]), L);
-        }
+  constexpr int per = 32 / G;
+  if constexpr (FX) {
+    if constexpr (G == 32) {
+      if (a.prefetch == 2) {
+        k_lap_one_tile<RR>(a, smem_raw + (size_t)wib * warp_smem_bytes_one(a.m), lane, warm,
+                           (long long)blockIdx.x * wpb + wib, nwarps);
+        return;
       }
     }
-    __syncwarp();
+    k_lap_prefetching<G, RR>(a, smem_raw + (size_t)wib * warp_smem_bytes_async(a.m, G), lane, warm,
+                             ((long long)blockIdx.x * wpb + wib) * per, nwarps * per);
+  } else {
+    const int grp = lane / G, gl = lane & (G - 1);
+    const int m = a.m, ld = tile_ld(m), mm = m * m;
+    unsigned char* base = smem_raw + (size_t)wib * warp_smem_bytes(m, G);
+    double* tile = reinterpret_cast<double*>(base) + (size_t)grp * m * ld;
+    double* uv = reinterpret_cast<double*>(base) + (size_t)per * m * ld;  // [0..31] u, [32..63] v
+    int* scr = reinterpret_cast<int*>(uv + 64) + grp * G;
+    unsigned long long aug_acc = 0, relax_acc = 0;
+    for (long long t0 = ((long long)blockIdx.x * wpb + wib) * per; t0 < a.batch; t0 += nwarps * per) {
+      const long long tb = t0 + grp;
+      const bool have = tb < a.batch;
+      const long long t = (have && a.map) ? (long long)a.map[tb] : tb;
+      stage_tile<G, false>(tile, ld, m, gl, have ? a.A + t * mm : nullptr, nullptr);
+      const double u0 = (warm && have && gl < m) ? a.u0[t * m + gl] : 0.0;
+      __syncwarp();
+      const WarpLapResult<double> R =
+          group_lap<G, true>(tile, ld, have ? m : 0, lane, warm, u0, a.dual_mode, scr, uv + grp * G);
+      if (have && gl < m) {
+        if (a.u) a.u[t * m + gl] = R.u;
+        if (a.v) a.v[t * m + gl] = R.v;
+        if (a.r2c) a.r2c[t * m + gl] = R.r2c;
+      }
+      if (have && gl == 0) {
+        a.value[t] = R.value;
+        if (a.naug) a.naug[t] = R.naug;
+        aug_acc += R.naug;
+        relax_acc += R.nrelax;
+      }
+      __syncwarp();
+    }
+    if (a.stats && gl == 0 && (aug_acc | relax_acc)) {
+      atomicAdd(a.stats + 0, aug_acc);
+      atomicAdd(a.stats + 1, relax_acc);
+    }
   }
-  if (a.stats && gl == 0 && (aug_acc | relax_acc)) {
-    atomicAdd(a.stats + 0, aug_acc);
-    atomicAdd(a.stats + 1, relax_acc);
+}
+
+// The Y and X stages: few LAPs whose latency is the stage's time, costs A + Badd
+// in, reduced costs out.  A block of four warps per LAP stages the tile (all of
+// a thread's loads in flight at once, the grid from a block maximum, converted
+// in registers) and writes the reduced costs; its first warp solves the LAP.
+// One warp per LAP spent 6 us of the X stage's 19 (n = 20) on staging.  n = 20: Y
+// 22.9 -> 17.9 us, X 19.1 -> 14.3; n = 12: 14.3 -> 12.7, 11.6 -> 9.7.
+constexpr int kBlockThreads = 128;
+template <bool FX, bool RR>
+__global__ void __launch_bounds__(kBlockThreads) k_lap_block(LapArgs a) {
+  if (a.skip && *a.skip) return;
+  using T = typename std::conditional<FX, long long, double>::type;
+  constexpr int kPer = 32 * 32 / kBlockThreads;  // entries of a thread, m = 32
+  __shared__ T tile[32 * 33];
+  __shared__ T uv[64];  // [0..31] u, [32..63] v
+  __shared__ int scr[32];
+  __shared__ unsigned top[kBlockThreads / 32];
+  const int tid = threadIdx.x, lane = tid & 31, m = a.m, ld = tile_ld(m), mm = m * m;
+  const long long t = a.map ? (long long)a.map[blockIdx.x] : (long long)blockIdx.x;
+  const bool warm = a.u0 != nullptr && (a.warm_gate == nullptr || *a.warm_gate != 0);
+  const double* src = a.A + t * mm;
+  const double* add = a.Badd ? a.Badd + t * mm : nullptr;
+  double x[kPer], y[kPer];
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) {
+    const int e = tid + k * kBlockThreads;
+    x[k] = e < mm ? __ldcs(src + e) : 0.0;
+    y[k] = (add && e < mm) ? __ldcs(add + e) : 0.0;
   }
+  const double u0d = (warm && tid < m) ? a.u0[t * m + tid] : 0.0;
+  unsigned eb = 0;
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) {
+    if (add) x[k] = __dadd_rn(x[k], y[k]);
+    if constexpr (FX) eb = max(eb, fx_expfield(x[k]));  // entries past the tile are 0
+  }
+  int L = 0;
+  if constexpr (FX) {
+    eb = __reduce_max_sync(kFull, eb);
+    if (lane == 0) top[tid >> 5] = eb;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < kBlockThreads / 32; ++w) eb = max(eb, top[w]);
+    L = fx_grid(eb);
+  }
+  // (r, c) of entry tid + k kBlockThreads, advanced without a division per entry
+  const int rq = kBlockThreads / m, cq = kBlockThreads - rq * m, r0 = tid / m, c0 = tid - r0 * m;
+  auto entries = [&](auto&& f) {
+    int r = r0, c = c0;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      if (tid + k * kBlockThreads < mm) f(k, r, c);
+      r += rq;
+      c += cq;
+      if (c >= m) {
+        c -= m;
+        ++r;
+      }
+    }
+  };
+  entries([&](int k, int r, int c) {
+    if constexpr (FX) tile[r * ld + c] = fx_floor(x[k], L, kFxEntryBits);
+    else tile[r * ld + c] = x[k];
+  });
+  __syncthreads();
+  if (tid < 32) {
+    WarpLapResult<T> R;
+    const T u0 = (warm && lane < m) ? start_dual<FX>(u0d, L) : T(0);
+    if constexpr (FX) R = group_lap_fx<32, RR>(tile, ld, m, lane, warm, u0, scr, uv);
+    else R = group_lap<32, false>(tile, ld, m, lane, warm, u0, a.dual_mode, scr, uv);
+    uv[lane] = R.u;
+    uv[32 + lane] = R.v;
+    if (lane < m) {
+      if (a.u) a.u[t * m + lane] = out_value<FX>(R.u, L);
+      if (a.v) a.v[t * m + lane] = out_value<FX>(R.v, L);
+      if (a.r2c) a.r2c[t * m + lane] = R.r2c;
+    }
+    if (lane == 0) {
+      a.value[t] = out_value<FX>(R.value, L);
+      if (a.naug) a.naug[t] = R.naug;
+      if (a.stats) {
+        atomicAdd(a.stats + 0, (unsigned long long)R.naug);
+        atomicAdd(a.stats + 1, (unsigned long long)R.nrelax);
+      }
+    }
+  }
+  if (!a.pi) return;
+  __syncthreads();
+  double* dst = a.pi + t * mm;
+  entries([&](int k, int r, int c) {
+    dst[tid + k * kBlockThreads] = out_value<FX>(lap_sub(lap_sub(tile[r * ld + c], uv[r]), uv[32 + c]), L);
+  });
+}
+
+cudaError_t launch_lap_blocks(const LapArgs& a, cudaStream_t s) {
+  if (a.batch <= 0) return cudaSuccess;
+  if (a.m < 1 || a.m > 32 || a.batch > 0x7fffffffll) return cudaErrorInvalidValue;
+  const int grid = (int)a.batch;
+  if (a.dual_mode != 1) k_lap_block<false, false><<<grid, kBlockThreads, 0, s>>>(a);
+  else if (a.u0) k_lap_block<true, false><<<grid, kBlockThreads, 0, s>>>(a);
+  else k_lap_block<true, true><<<grid, kBlockThreads, 0, s>>>(a);
+  return cudaGetLastError();
 }
 
 static int gidx(int G) { return G == 8 ? 0 : (G == 16 ? 1 : 2); }
 
 using LapKernel = void (*)(LapArgs);
 
-// The kernel for (group, in-place canonical pass, fixed-point arithmetic, row
-// reduction of cold starts; the last only with fixed point).
+// The forms of k_lap: FP64, fixed point, fixed point with the row reduction of
+// cold starts.
+constexpr int kForms = 3;
 template <int G>
-static LapKernel lap_kernel(bool pre, bool fx, bool rr) {
-  if (fx && rr) return pre ? k_lap<G, true, true, true> : k_lap<G, false, true, true>;
-  if (pre) return fx ? k_lap<G, true, true> : k_lap<G, true, false>;
-  return fx ? k_lap<G, false, true> : k_lap<G, false, false>;
+static LapKernel lap_kernel(int form) {
+  return form == 0 ? k_lap<G, false> : form == 1 ? k_lap<G, true> : k_lap<G, true, true>;
 }
-static LapKernel lap_kernel(int G, bool pre, bool fx, bool rr) {
-  return G == 8 ? lap_kernel<8>(pre, fx, rr) : (G == 16 ? lap_kernel<16>(pre, fx, rr) : lap_kernel<32>(pre, fx, rr));
+static LapKernel lap_kernel(int G, int form) {
+  return G == 8 ? lap_kernel<8>(form) : (G == 16 ? lap_kernel<16>(form) : lap_kernel<32>(form));
 }
-
-// The forms of k_lap: (pre, fx, rr) and, for the prefetching ones (fixed point,
-// no reduced-cost output), how the tile gets into shared memory.
-constexpr int kForms = 6;
-struct LapForm {
-  bool pre, fx, rr;
-};
-static LapForm lap_form(int k) { return LapForm{(k & 1) != 0, k >= 2, k >= 4}; }
-static int lap_form_index(bool pre, bool fx, bool rr) { return (rr ? 4 : (fx ? 2 : 0)) + (pre ? 1 : 0); }
+static int lap_form(const LapArgs& a) { return a.dual_mode != 1 ? 0 : (a.u0 ? 1 : 2); }
 
 // A launch of one form on the current device: its resident blocks and, for the
-// prefetching forms, a.prefetch (1 two tile buffers per warp, 2 the one-tile form).
+// fixed-point forms, a.prefetch (1 two tile buffers per warp, 2 the one-tile form).
 struct LapPlan {
   int occ = 0;  // resident blocks per SM, 0 = not configured
   int prefetch = 0;
@@ -332,7 +394,7 @@ static cudaError_t current_cfg(LapDevCfg** out) {
   return cudaSuccess;
 }
 
-// Every form of (G, m, wpb).  A prefetching form takes two tile buffers per
+// Every form of (G, m, wpb).  A fixed-point form takes two tile buffers per
 // warp unless one tile alone lets more warps onto an SM: m = 28 (16 -> 32
 // warps), not m = 18 (32 either way).
 static cudaError_t prepare_one(LapDevCfg& cfg, int G, int m, int wpb) {
@@ -341,8 +403,7 @@ static cudaError_t prepare_one(LapDevCfg& cfg, int G, int m, int wpb) {
   cudaError_t e;
   const int cap = (int)(warp_smem_bytes_async(32, 32) * kMaxWarpsPerBlock);
   for (int k = 0; k < kForms; ++k) {
-    const LapForm f = lap_form(k);
-    const LapKernel kern = lap_kernel(G, f.pre, f.fx, f.rr);
+    const LapKernel kern = lap_kernel(G, k);
     if (!cfg.attr[gidx(G)] &&
         (e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, cap)) != cudaSuccess)
       return e;
@@ -350,7 +411,7 @@ static cudaError_t prepare_one(LapDevCfg& cfg, int G, int m, int wpb) {
       return cudaOccupancyMaxActiveBlocksPerMultiprocessor(o, kern, wpb * 32, per_warp * wpb);
     };
     LapPlan p;
-    p.prefetch = f.pre && f.fx ? 1 : 0;
+    p.prefetch = k > 0 ? 1 : 0;
     p.smem = (p.prefetch ? warp_smem_bytes_async(m, G) : warp_smem_bytes(m, G)) * wpb;
     if ((e = occupancy(p.smem / wpb, &p.occ)) != cudaSuccess) return e;
     if (p.prefetch && G == 32) {
@@ -396,11 +457,12 @@ cudaError_t launch_lap(const LapArgs& a, cudaStream_t s) {
   if (a.batch <= 0) return cudaSuccess;
   const int G = a.group ? a.group : default_group(a.m);
   const int wpb = a.warps_per_block ? a.warps_per_block : kMaxWarpsPerBlock;
+  if (a.Badd || a.pi) return cudaErrorInvalidValue;  // launch_lap_blocks
   // a cold fixed-point launch reduces the rows first (the same canonical result)
-  const bool pre = a.pi == nullptr && a.Badd == nullptr, fx = a.dual_mode == 1, rr = fx && a.u0 == nullptr;
+  const int form = lap_form(a);
   LapPlan plan;
   long long cap = 0;
-  cudaError_t e = prepare_plan(a.m, G, wpb, lap_form_index(pre, fx, rr), &plan, &cap);
+  cudaError_t e = prepare_plan(a.m, G, wpb, form, &plan, &cap);
   if (e != cudaSuccess) return e;
   LapArgs b = a;
   b.prefetch = plan.prefetch;
@@ -417,7 +479,7 @@ cudaError_t launch_lap(const LapArgs& a, cudaStream_t s) {
     b.fixed_part = a.batch / round / 2 * round;
     if (!b.head_zeroed && (e = cudaMemsetAsync(b.head, 0, sizeof(unsigned long long), s)) != cudaSuccess) return e;
   }
-  lap_kernel(G, pre, fx, rr)<<<grid, wpb * 32, plan.smem, s>>>(b);
+  lap_kernel(G, form)<<<grid, wpb * 32, plan.smem, s>>>(b);
   return cudaGetLastError();
 }
 
@@ -425,7 +487,7 @@ bool lap_wants_queue(long long batch, int m) {
   LapPlan plan;
   long long cap = 0;
   const int G = default_group(m);
-  if (prepare_plan(m, G, kMaxWarpsPerBlock, lap_form_index(true, true, false), &plan, &cap) != cudaSuccess) return false;
+  if (prepare_plan(m, G, kMaxWarpsPerBlock, 1, &plan, &cap) != cudaSuccess) return false;
   return batch > cap * kMaxWarpsPerBlock * (32 / G);
 }
 

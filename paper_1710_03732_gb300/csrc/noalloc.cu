@@ -191,7 +191,7 @@ extern "C" rlt2_status rlt2_iterate_noalloc(int n, const double* F, const double
   if ((e = cudaMemcpyAsync(v.xcost, v.bprime, sizeof(double) * n2, cudaMemcpyDeviceToDevice, s)) != cudaSuccess ||
       (e = cudaMemcpyAsync(&v.sc->lb_base, v.d_cst, sizeof(double), cudaMemcpyDeviceToDevice, s)) != cudaSuccess)
     return cuda_fail(e, "rlt2_iterate_noalloc: x costs");
-  if ((e = prepare_lap_stages(n)) != cudaSuccess) return cuda_fail(e, "rlt2_iterate_noalloc: prepare");
+  if ((e = prepare_lap(n - 2)) != cudaSuccess) return cuda_fail(e, "rlt2_iterate_noalloc: prepare");
   for (int it = 0; it < iters; ++it)
     if ((e = enqueue_iteration(v, s, nullptr)) != cudaSuccess) return cuda_fail(e, "rlt2_iterate_noalloc: iterate");
   return RLT2_OK;

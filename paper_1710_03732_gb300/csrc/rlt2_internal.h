@@ -150,11 +150,12 @@ int default_group(int m);
 // outside stream capture before the first launch of that size.
 cudaError_t prepare_lap(int m, int group = 0, int warps_per_block = 0);
 
-// The same for the three LAP stages of an n-facility iteration (ascent.cu).
-cudaError_t prepare_lap_stages(int n);
-
 // Enqueue the batched LAP kernel (grid sized for the device); returns the CUDA error.
+// Without Badd and pi.
 cudaError_t launch_lap(const LapArgs& a, cudaStream_t s);
+// One block per LAP, with Badd and pi (the Y and X stages; head, group and
+// warps_per_block unused).
+cudaError_t launch_lap_blocks(const LapArgs& a, cudaStream_t s);
 
 // Whether a fixed-point batch of the default shape is more than its resident
 // warps hold at once, so that launch_lap would use a queue (LapArgs::head).
