@@ -103,6 +103,7 @@ static const int h_widx[5] = {0, 1, 3, 2, 4};
 
 // blockDim.x a multiple of 32 (the folded form's warps move 32 tiles together)
 __global__ void k_move_y(MoveYArgs a) {
+  dependent_begin();
   // the Z stage's launch comes after this one on the stream
   if (a.lap_head && blockIdx.x == 0 && threadIdx.x == 0) *a.lap_head = 0;
   if (!a.sc->have_snap || a.sc->done) return;
@@ -113,6 +114,7 @@ __global__ void k_move_y(MoveYArgs a) {
 
 // at most 352 threads (move_z_threads) and 62 registers: three blocks per SM
 __global__ void __launch_bounds__(352, 3) k_move_z(MoveZArgs a) {
+  dependent_begin();
   if (!a.sc->have_snap || a.sc->done) return;
   move_z_block(a, blockIdx.x, threadIdx.x, blockDim.x);
 }
@@ -123,6 +125,7 @@ __global__ void __launch_bounds__(352, 3) k_move_z(MoveZArgs a) {
 // for the FP64 form.  What bounds it: the L2 tags (73 % busy, a request per
 // segment), then the FP64 pipe (54 %) and the ALU pipe (42 %).
 __global__ void __launch_bounds__(256, 4) k_move_z_fixed(MoveZArgs a) {
+  dependent_begin();
   if (!a.sc->have_snap || a.sc->done) return;
   const int w = blockIdx.x * 8 + (threadIdx.x >> 5);
   if (w < fixed_warps(a.n)) move_z_fixed_warp(a, blockIdx.y, w, threadIdx.x & 31);
@@ -131,6 +134,7 @@ __global__ void __launch_bounds__(256, 4) k_move_z_fixed(MoveZArgs a) {
 // Second phase of the two-phase Z solve; runs on every iteration (the first
 // phase's duals are always fresh).
 __global__ void __launch_bounds__(512) k_phase2(Phase2Args a) {
+  dependent_begin();
   if (a.sc->done) return;
   phase2_block(a, blockIdx.x);
 }
@@ -148,6 +152,7 @@ __global__ void k_pi_z(long long E, int m, const double* Dhat, const double* xi,
 
 // ---------------------------------------------------------------- finalize ----
 __global__ void __launch_bounds__(256) k_finalize(FinArgs a) {
+  dependent_begin();
   if (a.sc->done) return;
   finalize_block(a);
 }
@@ -937,20 +942,21 @@ cudaError_t rlt2::enqueue_iteration(const IterView& v, cudaStream_t s, cudaEvent
     const MoveYArgs my = make_move_y(v);
     const long long blocks = (T + 255) / 256;
     k_move_y<<<(int)(blocks < 8192 ? blocks : 8192), 256, 0, s>>>(my);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     count(0, 1);
   }
-  if ((e = cudaGetLastError()) != cudaSuccess || (e = rec(0, 1)) != cudaSuccess) return e;
+  if ((e = rec(0, 1)) != cudaSuccess) return e;
   // 2) z move (inside the Z-stage launch when pipelined)
   const MoveZArgs mz = make_move_z(v);
   const bool pipelined = v.pplan && v.pipe && !p.half_z && p.warm != 2;
   if ((e = rec(1, 0)) != cudaSuccess) return e;
   if (!pipelined) {
     if (mz.fixed)
-      k_move_z_fixed<<<dim3((fixed_warps(n) + 7) / 8, v.ntrip), 256, 0, s>>>(mz);
+      e = launch_dependent(k_move_z_fixed, dim3((fixed_warps(n) + 7) / 8, v.ntrip), 256, 0, s, mz);
     else  // one thread per (q, r) class of the block's (triple, p): round to whole warps
-      k_move_z<<<v.ntrip * n, move_z_threads(n), 0, s>>>(mz);
+      e = launch_dependent(k_move_z, v.ntrip * n, move_z_threads(n), 0, s, mz);
+    if (e != cudaSuccess) return e;
     count(1, 1);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   if ((e = rec(1, 1)) != cudaSuccess) return e;
   // 3) Z stage
@@ -988,9 +994,8 @@ cudaError_t rlt2::enqueue_iteration(const IterView& v, cudaStream_t s, cudaEvent
   // 3b) two-phase Z solve: move slack onto the zero-slack members, solve again
   if ((e = rec(6, 0)) != cudaSuccess) return e;
   if (p.two_phase) {
-    k_phase2<<<v.ntrip * n, move_z_threads(n), 0, s>>>(make_phase2(v));
+    if ((e = launch_dependent(k_phase2, v.ntrip * n, move_z_threads(n), 0, s, make_phase2(v))) != cudaSuccess) return e;
     count(6, 1);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   if ((e = rec(6, 1)) != cudaSuccess || (e = rec(7, 0)) != cudaSuccess) return e;
   if (p.two_phase) {
@@ -1044,9 +1049,9 @@ cudaError_t rlt2::enqueue_iteration(const IterView& v, cudaStream_t s, cudaEvent
   // 6) finalize
   const FinArgs f = make_fin(v);
   if ((e = rec(5, 0)) != cudaSuccess) return e;
-  k_finalize<<<1, 256, 0, s>>>(f);
+  if ((e = launch_dependent(k_finalize, 1, 256, 0, s, f)) != cudaSuccess) return e;
   count(5, 1);
-  if ((e = cudaGetLastError()) != cudaSuccess || (e = rec(5, 1)) != cudaSuccess) return e;
+  if ((e = rec(5, 1)) != cudaSuccess) return e;
   return cudaSuccess;
 }
 

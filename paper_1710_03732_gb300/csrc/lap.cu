@@ -187,6 +187,7 @@ constexpr int kLapBlocks = G == 16 ? 3 : 4;
 // (fixed point, cold launches) reduces the rows of a cold start first.
 template <int G, bool FX, bool RR = false>
 __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32, kLapBlocks<G>) k_lap(LapArgs a) {
+  dependent_begin();
   if (a.skip && *a.skip) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, wpb = blockDim.x >> 5;
@@ -249,6 +250,7 @@ __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32, kLapBlocks<G>) k_lap(L
 constexpr int kBlockThreads = 128;
 template <bool FX, bool RR>
 __global__ void __launch_bounds__(kBlockThreads) k_lap_block(LapArgs a) {
+  dependent_begin();
   if (a.skip && *a.skip) return;
   using T = typename std::conditional<FX, long long, double>::type;
   constexpr int kPer = 32 * 32 / kBlockThreads;  // entries of a thread, m = 32
@@ -333,19 +335,18 @@ __global__ void __launch_bounds__(kBlockThreads) k_lap_block(LapArgs a) {
   });
 }
 
+using LapKernel = void (*)(LapArgs);
+
 cudaError_t launch_lap_blocks(const LapArgs& a, cudaStream_t s) {
   if (a.batch <= 0) return cudaSuccess;
   if (a.m < 1 || a.m > 32 || a.batch > 0x7fffffffll) return cudaErrorInvalidValue;
   const int grid = (int)a.batch;
-  if (a.dual_mode != 1) k_lap_block<false, false><<<grid, kBlockThreads, 0, s>>>(a);
-  else if (a.u0) k_lap_block<true, false><<<grid, kBlockThreads, 0, s>>>(a);
-  else k_lap_block<true, true><<<grid, kBlockThreads, 0, s>>>(a);
-  return cudaGetLastError();
+  const LapKernel kern =
+      a.dual_mode != 1 ? k_lap_block<false, false> : (a.u0 ? k_lap_block<true, false> : k_lap_block<true, true>);
+  return launch_dependent(kern, grid, kBlockThreads, 0, s, a);
 }
 
 static int gidx(int G) { return G == 8 ? 0 : (G == 16 ? 1 : 2); }
-
-using LapKernel = void (*)(LapArgs);
 
 // The forms of k_lap: FP64, fixed point, fixed point with the row reduction of
 // cold starts.
@@ -479,6 +480,7 @@ cudaError_t launch_lap(const LapArgs& a, cudaStream_t s) {
     b.fixed_part = a.batch / round / 2 * round;
     if (!b.head_zeroed && (e = cudaMemsetAsync(b.head, 0, sizeof(unsigned long long), s)) != cudaSuccess) return e;
   }
+  if (a.dependent) return launch_dependent(lap_kernel(G, form), grid, wpb * 32, plan.smem, s, b);
   lap_kernel(G, form)<<<grid, wpb * 32, plan.smem, s>>>(b);
   return cudaGetLastError();
 }
@@ -796,6 +798,7 @@ extern "C" rlt2_status rlt2_lap_batched(int batch, int m, const double* cost, co
     (void)cudaGetLastError();
   }
   a.head = head;
+  a.dependent = 1;  // small batches back to back: 400 LAPs of size 7 14.7 -> 12.8 us a call
   cudaError_t e = launch_lap(a, s);
   if (head) {
     const cudaError_t ef = cudaFreeAsync(head, s);

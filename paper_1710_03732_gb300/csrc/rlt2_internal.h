@@ -42,6 +42,38 @@ unsigned long long oob_ascent();
 unsigned long long oob_nodes();
 unsigned long long oob_fused();
 
+// Programmatic dependent launch (host side below): a kernel launched with
+// launch_dependent may start while the kernel before it on the stream is still
+// running; dependent_begin() lets its own successor start in the same way and
+// then waits until everything before it has finished and is visible.  Called
+// first thing by every thread, before any global memory is touched, it leaves
+// the order that the stream gives; what overlaps is the launch itself.  In an
+// iteration the z move, the Y and X stages and k_finalize are launched this way
+// (kernel by kernel n = 8 45 -> 38 us per iteration, n = 12 78 -> 71, n = 20
+// 704 -> 697; in graph replay, whose gaps are short already, 31.3 and 31.0,
+// 66); k_move_y and the Z stage normally: the z move's blocks, resident and
+// waiting since before k_move_y began, made it 170 us longer at n = 20.
+#ifdef __CUDACC__
+__device__ __forceinline__ void dependent_begin() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+template <typename... P, typename... A>
+cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, P(args)...);
+}
+#endif
+
 struct MoveZArgs;
 struct DevScalars;
 
@@ -70,6 +102,7 @@ struct LapArgs {
                              // the next tile by cp.async while it solves the current one
   unsigned long long* head;  // nullable: device counter of the prefetching form's LAP queue
                              // (launch_lap zeroes it on the stream before the launch)
+  int dependent;             // launched as a programmatic dependent (see launch_dependent)
   int head_zeroed;           // an earlier launch on the stream has zeroed *head: no memset
 };
 
