@@ -27,6 +27,7 @@
 // make every kernel a no-op after a stop, so whole batches of iterations can
 // be enqueued without host round trips.
 #include <cmath>
+#include <cstdint>
 #include <cstdio>
 #include <cstring>
 #include <mutex>
@@ -112,31 +113,29 @@ __global__ void k_move_y(MoveYArgs a) {
   else move_y_range(a, start, stride);
 }
 
-// at most 352 threads (move_z_threads) and 62 registers: three blocks per SM
-__global__ void __launch_bounds__(352, 3) k_move_z(MoveZArgs a) {
-  dependent_begin();
-  if (!a.sc->have_snap || a.sc->done) return;
-  move_z_block(a, blockIdx.x, threadIdx.x, blockDim.x);
-}
-
-// The integer form of the folded move: blockIdx.y = triple, eight of its warps
-// per block.  Four blocks per SM at 64 registers: 0.291 ms at n = 20 (two to
-// five blocks 0.309, 0.309, 0.293), 3.72 ms at n = 30, against 0.461 and 6.3 ms
-// for the FP64 form.  What bounds it: the L2 tags (73 % busy, a request per
-// segment), then the FP64 pipe (54 %) and the ALU pipe (42 %).
-__global__ void __launch_bounds__(256, 4) k_move_z_fixed(MoveZArgs a) {
+// blockIdx.y = triple, eight of its warps per block; FIXED: the integer form of
+// the folded move.  Four blocks per SM at 64 registers.  Integer form: 0.291 ms at
+// n = 20 (two to five blocks 0.309, 0.309, 0.293), 3.72 ms at n = 30, against
+// 0.461 and 6.3 ms for the FP64 form; bound by the L2 tags (73 % busy, a request
+// per segment), then the FP64 pipe (54 %) and the ALU pipe (42 %).  FP64 form:
+// n = 20 folded 461 -> 454 us with these lanes, n = 16 126 -> 120.
+template <bool FIXED>
+__global__ void __launch_bounds__(256, 4) k_move_z(MoveZArgs a) {
   dependent_begin();
   if (!a.sc->have_snap || a.sc->done) return;
   const int w = blockIdx.x * 8 + (threadIdx.x >> 5);
-  if (w < fixed_warps(a.n)) move_z_fixed_warp(a, blockIdx.y, w, threadIdx.x & 31);
+  if (w < class_warps(a.n)) move_z_warp<FIXED>(a, blockIdx.y, w, threadIdx.x & 31);
 }
 
 // Second phase of the two-phase Z solve; runs on every iteration (the first
-// phase's duals are always fresh).
-__global__ void __launch_bounds__(512) k_phase2(Phase2Args a) {
+// phase's duals are always fresh).  Bound by the FP64 pipe: most members are
+// told apart by exponents (in_basis), four FP64 operations each instead of seven.
+// With the FP64 move's lanes, 30 F two-phase iterations at n = 16 30.7 -> 28.8 ms.
+__global__ void __launch_bounds__(256, 4) k_phase2(Phase2Args a) {
   dependent_begin();
   if (a.sc->done) return;
-  phase2_block(a, blockIdx.x);
+  const int w = blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (w < class_warps(a.n)) phase2_warp(a, blockIdx.y, w, threadIdx.x & 31);
 }
 
 // pi_z = (D^ - xi_k') - psi_r' for every z entry (reduced costs on demand).
@@ -853,6 +852,10 @@ Phase2Args rlt2::make_phase2(const IterView& v) {
   a.n = v.n;
   a.m = v.m;
   a.tol = v.prm.phase2_tol;
+  std::uint64_t bits;
+  std::memcpy(&bits, &a.tol, sizeof bits);
+  a.tol_exp = (int)((bits >> 52) & 0x7ff) - 1023;
+  a.rcp = class_rcp(v.n);
   a.Dhat = v.Dhat;
   a.xi = v.xi;
   a.psi = v.psi;
@@ -879,8 +882,7 @@ MoveZArgs rlt2::make_move_z(const IterView& v) {
   // the move need not follow the FP64 rounding order of modes 0 and 2
   mz.fixed = mz.folded && p.dual_mode == 1;
   mz.phi_fx = fx_factor(p.phi_z[0]);
-  mz.rcp_groups = (unsigned)(((1ull << 31) + fixed_groups(v.n) - 1) / fixed_groups(v.n));
-  mz.rcp_8m = (unsigned)(((1ull << 31) + 8 * v.m - 1) / (8 * v.m));
+  mz.rcp = class_rcp(v.n);
   mz.saterm = v.saterm;
   mz.Dhat = v.Dhat;
   mz.xi = v.xi;
@@ -948,13 +950,11 @@ cudaError_t rlt2::enqueue_iteration(const IterView& v, cudaStream_t s, cudaEvent
   if ((e = rec(0, 1)) != cudaSuccess) return e;
   // 2) z move (inside the Z-stage launch when pipelined)
   const MoveZArgs mz = make_move_z(v);
+  const dim3 class_grid((class_warps(n) + 7) / 8, v.ntrip);
   const bool pipelined = v.pplan && v.pipe && !p.half_z && p.warm != 2;
   if ((e = rec(1, 0)) != cudaSuccess) return e;
   if (!pipelined) {
-    if (mz.fixed)
-      e = launch_dependent(k_move_z_fixed, dim3((fixed_warps(n) + 7) / 8, v.ntrip), 256, 0, s, mz);
-    else  // one thread per (q, r) class of the block's (triple, p): round to whole warps
-      e = launch_dependent(k_move_z, v.ntrip * n, move_z_threads(n), 0, s, mz);
+    e = launch_dependent(mz.fixed ? k_move_z<true> : k_move_z<false>, class_grid, 256, 0, s, mz);
     if (e != cudaSuccess) return e;
     count(1, 1);
   }
@@ -994,7 +994,7 @@ cudaError_t rlt2::enqueue_iteration(const IterView& v, cudaStream_t s, cudaEvent
   // 3b) two-phase Z solve: move slack onto the zero-slack members, solve again
   if ((e = rec(6, 0)) != cudaSuccess) return e;
   if (p.two_phase) {
-    if ((e = launch_dependent(k_phase2, v.ntrip * n, move_z_threads(n), 0, s, make_phase2(v))) != cudaSuccess) return e;
+    if ((e = launch_dependent(k_phase2, class_grid, 256, 0, s, make_phase2(v))) != cudaSuccess) return e;
     count(6, 1);
   }
   if ((e = rec(6, 1)) != cudaSuccess || (e = rec(7, 0)) != cudaSuccess) return e;

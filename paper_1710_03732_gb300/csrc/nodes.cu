@@ -38,27 +38,22 @@ __global__ void k_move_y_nodes(const MoveYArgs* nodes) {
   else move_y_range(a, start, stride);
 }
 
-__global__ void __launch_bounds__(352, 3) k_move_z_nodes(const MoveZArgs* nodes, const int* nblocks) {
-  if ((int)blockIdx.x >= nblocks[blockIdx.y]) return;
-  const MoveZArgs a = nodes[blockIdx.y];
-  if (!a.sc->have_snap || a.sc->done) return;
-  move_z_block(a, blockIdx.x, threadIdx.x, blockDim.x);
-}
-
-// The integer form: blockIdx.y = triple, blockIdx.z = node.
-__global__ void __launch_bounds__(256, 4) k_move_z_fixed_nodes(const MoveZArgs* nodes, const int* nblocks) {
+// blockIdx.y = triple, blockIdx.z = node, eight of the triple's warps per block.
+template <bool FIXED>
+__global__ void __launch_bounds__(256, 4) k_move_z_nodes(const MoveZArgs* nodes, const int* ntrips) {
   const MoveZArgs& a = nodes[blockIdx.z];
   const int w = blockIdx.x * 8 + (threadIdx.x >> 5);
-  if ((int)blockIdx.y * a.n >= nblocks[blockIdx.z] || w >= fixed_warps(a.n)) return;
+  if ((int)blockIdx.y >= ntrips[blockIdx.z] || w >= class_warps(a.n)) return;
   if (!a.sc->have_snap || a.sc->done) return;
-  move_z_fixed_warp(a, blockIdx.y, w, threadIdx.x & 31);
+  move_z_warp<FIXED>(a, blockIdx.y, w, threadIdx.x & 31);
 }
 
-__global__ void __launch_bounds__(512) k_phase2_nodes(const Phase2Args* nodes, const int* nblocks) {
-  if ((int)blockIdx.x >= nblocks[blockIdx.y]) return;
-  const Phase2Args a = nodes[blockIdx.y];
+__global__ void __launch_bounds__(256, 4) k_phase2_nodes(const Phase2Args* nodes, const int* ntrips) {
+  const Phase2Args& a = nodes[blockIdx.z];
+  const int w = blockIdx.x * 8 + (threadIdx.x >> 5);
+  if ((int)blockIdx.y >= ntrips[blockIdx.z] || w >= class_warps(a.n)) return;
   if (a.sc->done) return;
-  phase2_block(a, blockIdx.x);
+  phase2_warp(a, blockIdx.y, w, threadIdx.x & 31);
 }
 
 __global__ void __launch_bounds__(256) k_finalize_nodes(const FinArgs* nodes) {
@@ -155,7 +150,7 @@ struct WaveDev {
   MoveYArgs* my = nullptr;
   MoveZArgs* mz = nullptr;
   Phase2Args* p2 = nullptr;
-  int* mz_blocks = nullptr;
+  int* mz_trips = nullptr;
   FinArgs* fin = nullptr;
   unsigned long long* heads = nullptr;  // [kStages][kMaxRuns]
   unsigned long long* stats = nullptr;  // [6]
@@ -179,7 +174,7 @@ struct Wave {
   int cold = 0;  // warm == 0: no LAP of the wave has start duals
   long long total[kStages] = {0, 0, 0, 0};
   int max_m[kStages] = {0, 0, 0, 0};
-  int max_blocks = 0;
+  int max_trips = 0;
   int max_T = 0;
   int max_n = 0;
   std::vector<int> zm;     // Z-LAP size of each sorted Z item
@@ -254,11 +249,9 @@ cudaError_t enqueue_wave_iteration(const Wave& w, const WaveDev& d, int dual_mod
     k_move_y_nodes<<<dim3(bx, w.nn), 256, 0, s>>>(d.my);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
-  if (w.fixed)
-    k_move_z_fixed_nodes<<<dim3((fixed_warps(w.max_n) + 7) / 8, w.max_blocks / w.max_n, w.nn), 256, 0, s>>>(
-        d.mz, d.mz_blocks);
-  else
-    k_move_z_nodes<<<dim3(w.max_blocks, w.nn), move_z_threads(w.max_n), 0, s>>>(d.mz, d.mz_blocks);
+  const dim3 class_grid((class_warps(w.max_n) + 7) / 8, w.max_trips, w.nn);
+  if (w.fixed) k_move_z_nodes<true><<<class_grid, 256, 0, s>>>(d.mz, d.mz_trips);
+  else k_move_z_nodes<false><<<class_grid, 256, 0, s>>>(d.mz, d.mz_trips);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   for (const LearnedStart& ls : w.learned)
     if ((e = mlp_predict_enqueue(w.mlp, ls.T, ls.m, ls.Dhat, ls.xi, ls.u0, s)) != cudaSuccess) return e;
@@ -269,7 +262,7 @@ cudaError_t enqueue_wave_iteration(const Wave& w, const WaveDev& d, int dual_mod
     const int stage = order[oi];
     if (stage == 3) {
       if (!w.two_phase) continue;
-      k_phase2_nodes<<<dim3(w.max_blocks, w.nn), move_z_threads(w.max_n), 0, s>>>(d.p2, d.mz_blocks);
+      k_phase2_nodes<<<class_grid, 256, 0, s>>>(d.p2, d.mz_trips);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     NodeLapArgs a{};
@@ -374,9 +367,9 @@ void add_node(Wave& w, WaveHost& h, int j, const IterView& v, const rlt2_params&
   h.mz[j] = make_move_z(v);
   w.fixed = w.fixed && h.mz[j].fixed;
   h.p2[j] = make_phase2(v);
-  h.mzb[j] = v.ntrip * nr;
+  h.mzb[j] = v.ntrip;
   h.fin[j] = make_fin(v);
-  w.max_blocks = std::max(w.max_blocks, h.mzb[j]);
+  w.max_trips = std::max(w.max_trips, h.mzb[j]);
   w.max_T = std::max(w.max_T, (int)v.T);
   w.max_n = std::max(w.max_n, nr);
 }
@@ -407,7 +400,7 @@ cudaError_t upload_wave(const Wave& w, const WaveHost& h, const WaveDev& d, cuda
       (e = cudaMemcpyAsync(d.my, h.my.data(), sizeof(MoveYArgs) * w.nn, cudaMemcpyHostToDevice, s)) != cudaSuccess ||
       (e = cudaMemcpyAsync(d.mz, h.mz.data(), sizeof(MoveZArgs) * w.nn, cudaMemcpyHostToDevice, s)) != cudaSuccess ||
       (e = cudaMemcpyAsync(d.p2, h.p2.data(), sizeof(Phase2Args) * w.nn, cudaMemcpyHostToDevice, s)) != cudaSuccess ||
-      (e = cudaMemcpyAsync(d.mz_blocks, h.mzb.data(), sizeof(int) * w.nn, cudaMemcpyHostToDevice, s)) !=
+      (e = cudaMemcpyAsync(d.mz_trips, h.mzb.data(), sizeof(int) * w.nn, cudaMemcpyHostToDevice, s)) !=
           cudaSuccess ||
       (e = cudaMemcpyAsync(d.fin, h.fin.data(), sizeof(FinArgs) * w.nn, cudaMemcpyHostToDevice, s)) != cudaSuccess)
     return e;
@@ -421,7 +414,7 @@ cudaError_t alloc_wave_dev(WaveDev& d) {
       (e = cudaMalloc((void**)&d.my, sizeof(MoveYArgs) * kMaxWaveNodes)) != cudaSuccess ||
       (e = cudaMalloc((void**)&d.mz, sizeof(MoveZArgs) * kMaxWaveNodes)) != cudaSuccess ||
       (e = cudaMalloc((void**)&d.p2, sizeof(Phase2Args) * kMaxWaveNodes)) != cudaSuccess ||
-      (e = cudaMalloc((void**)&d.mz_blocks, sizeof(int) * kMaxWaveNodes)) != cudaSuccess ||
+      (e = cudaMalloc((void**)&d.mz_trips, sizeof(int) * kMaxWaveNodes)) != cudaSuccess ||
       (e = cudaMalloc((void**)&d.fin, sizeof(FinArgs) * kMaxWaveNodes)) != cudaSuccess ||
       (e = cudaMalloc((void**)&d.heads, sizeof(unsigned long long) * kStages * kMaxRuns)) != cudaSuccess ||
       (e = cudaMalloc((void**)&d.stats, sizeof(unsigned long long) * 6)) != cudaSuccess ||
@@ -431,7 +424,7 @@ cudaError_t alloc_wave_dev(WaveDev& d) {
 }
 
 void free_wave_dev(WaveDev& d) {
-  void* frees[] = {d.items, d.prefix, d.my, d.mz, d.p2, d.mz_blocks, d.fin, d.heads, d.stats, d.live};
+  void* frees[] = {d.items, d.prefix, d.my, d.mz, d.p2, d.mz_trips, d.fin, d.heads, d.stats, d.live};
   for (void* q : frees)
     if (q) cudaFree(q);
   d = WaveDev{};

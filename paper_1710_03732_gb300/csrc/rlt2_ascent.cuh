@@ -172,6 +172,11 @@ __device__ __forceinline__ void move_y_shift_range(const MoveYArgs& a, long long
   constexpr int kPart[6][5] = {{1, 2, 3, 4, 5}, {0, 4, 5, 2, 3}, {3, 0, 1, 5, 4},                    \
                                {2, 5, 4, 0, 1}, {5, 1, 0, 3, 2}, {4, 3, 2, 1, 0}};
 
+// ceil(2^31 / d) for d = class_groups(n) and 8 m: exact quotients while x d < 2^31.
+struct ClassRcp {
+  unsigned groups, m8;
+};
+
 struct MoveZArgs {
   int n, m;
   double kz;
@@ -185,7 +190,7 @@ struct MoveZArgs {
   double c1;
   int fixed;        // folded move in integers (canonical duals in fixed point; see rlt2_movefx.cuh)
   FxFactor phi_fx;  // phi of the fixed form
-  unsigned rcp_groups, rcp_8m;  // ceil(2^31 / d), d = fixed_groups(n) and 8 m: exact quotients while x d < 2^31
+  ClassRcp rcp;
   const double* saterm;  // n*n Type 4 amounts (F variant, when sc->sa_on)
   double* Dhat;
   const double* xi;
@@ -194,80 +199,6 @@ struct MoveZArgs {
   const int* trips;  // i | j<<8 | k<<16 with i<j<k
   const DevScalars* sc;
 };
-
-// The class (q, r) -- as indices qq < n-1, rr < n-2 with p (and q) skipped --
-// of thread slot c of a (triple, p) block.  Two members of a class lie in rows
-// along r, two in rows along q and two in a different tile for every (q, r):
-// with lanes along r (slot c = qq (n-2) + rr) a warp's six loads touch 144
-// 32-byte sectors.  For n >= 22 the slots run in bands of eight q with r
-// outer, so a warp's lanes cover 8 q x 4 r and touch 96: the z array is then
-// far larger than L2 and the move keeps its rate (n = 28: 3.60 instead of
-// 5.58 ms).  Below that the plain order is as fast or faster (n = 20 equal,
-// the batched nodes of residual 14..18 9 % faster without the bands' integer
-// divisions).
-template <bool BAND = true>
-__device__ __forceinline__ void class_of(int c, int n1, int m, int& qq, int& rr) {
-  constexpr int kBand = 8;
-  if (!BAND || n1 < 21) {
-    qq = c / m;
-    rr = c - qq * m;
-    return;
-  }
-  const int band = c / (kBand * m), cb = c - band * kBand * m;
-  const int hb = min(kBand, n1 - kBand * band);
-  qq = kBand * band + cb % hb;
-  rr = cb / hb;
-}
-
-// One thread per class; a block covers one facility triple and one location p
-// of its first facility (all (q, r)).  Consecutive threads take consecutive r,
-// so members (i,j,k|p,q,r) and (j,i,k|q,p,r) are read and written as contiguous
-// rows; the other four members' rows are shared by the block or by the n blocks
-// of the same triple, which run back to back.
-// Half-Z scheme (Section 5): the upper members (i,j,k|p,q,r), (i,k,j|p,r,q) and
-// (j,k,i|q,r,p) -- members 0, 1, 3 -- pool s = kz pi_z + tile term and each
-// receives half of the other two pools: D' = D - s + (S - s)/2 with S the sum
-// of the three pools in member order, evaluated as fma(-3/2, s, fma(1/2, S, D)).
-// Lower members are never touched.
-__device__ __forceinline__ void move_z_half_block(const MoveZArgs& a, int blk) {
-  RLT2_CLASS_TABLES
-  (void)kPart;
-  constexpr int kUp[3] = {0, 1, 3};
-  const int n = a.n, m = a.m, n1 = n - 1;
-  const int tr = blk / n, p = blk - tr * n;
-  const int packed = a.trips[tr];
-  const int F3[3] = {packed & 255, (packed >> 8) & 255, packed >> 16};
-  const int npairs = n1 * m;
-  const long long mm = (long long)m * m;
-  for (int c = threadIdx.x; c < npairs; c += blockDim.x) {
-    int qq, rr;
-    class_of(c, n1, m, qq, rr);
-    const int q = qq + (qq >= p);
-    const int lo = p < q ? p : q, hi = p < q ? q : p;
-    int r = rr;
-    r += (r >= lo);
-    r += (r >= hi);
-    const int L3[3] = {p, q, r};
-    double s[3], Dv[3];
-    long long idx[3];
-#pragma unroll
-    for (int u = 0; u < 3; ++u) {
-      const int b = kUp[u];
-      const int f0 = F3[kOrd[b][0]], f1 = F3[kOrd[b][1]], f2 = F3[kOrd[b][2]];
-      const int l0 = L3[kOrd[b][0]], l1 = L3[kOrd[b][1]], l2 = L3[kOrd[b][2]];
-      const long long t = RLT2_IDX(((long long)(f0 * n + l0) * n1 + (f1 - (f1 > f0))) * n1 + (l1 - (l1 > l0)),
-                                        (long long)n * n * n1 * n1);
-      const int kr = RLT2_IDX(f2 - (f2 > f0) - (f2 > f1), m), cc = RLT2_IDX(l2 - (l2 > l0) - (l2 > l1), m);
-      idx[u] = t * mm + kr * m + cc;
-      Dv[u] = a.Dhat[idx[u]];
-      const double pz = dsub_(dsub_(Dv[u], __ldg(a.xi + t * m + kr)), __ldg(a.psi + t * m + cc));
-      s[u] = a.kz_one ? dadd_(pz, __ldg(a.tterm + t)) : __fma_rn(a.kz, pz, __ldg(a.tterm + t));
-    }
-    const double S = dadd_(dadd_(s[0], s[1]), s[2]);
-#pragma unroll
-    for (int u = 0; u < 3; ++u) a.Dhat[idx[u]] = __fma_rn(-1.5, s[u], __fma_rn(0.5, S, Dv[u]));
-  }
-}
 
 // Loads of the duals and tile terms: through the read-only cache in the
 // stand-alone move; plain loads where the same launch later rewrites the duals
@@ -279,31 +210,48 @@ __device__ __forceinline__ double ldv(const double* p) {
   else return *p;
 }
 
-// The folded move of the class {(i,p),(j,q),(k,r)}, i < j < k, in the integer
-// form; cr is r's position among the locations without p and q.  Member order
-// and indices are those of RLT2_CLASS_TABLES, written out so that what does not
-// depend on the locations is formed once per block: 32-bit indices (at most
-// 885,657,600 entries for n = 32).
-template <bool RO>
-__device__ __forceinline__ void move_class_fixed(const MoveZArgs& a, int i, int j, int k, int p, int q, int r, int cr) {
-  const unsigned n = a.n, m = a.m, n1 = n - 1, n2 = n1 * n1;
+// Where the members of the class {(i,p),(j,q),(k,r)}, i < j < k, lie: member b's
+// entry at[b] of D^, its row dual xi[tm[b] + row[b]], column dual psi[tm[b] +
+// col[b]], tile t[b] and (first facility, first location) fl[b].  Member order as
+// in kOrd, written out so that what does not depend on the locations is formed
+// once per block; cr is r's position among the locations without p and q.
+// 32-bit indices (at most 885,657,600 entries for n = 32).
+struct ClassIdx {
+  unsigned t[6], tm[6], row[6], col[6], at[6], fl[6];
+};
+__device__ __forceinline__ ClassIdx class_idx(unsigned n, unsigned m, int i, int j, int k, int p, int q, int r,
+                                              int cr) {
+  const unsigned n1 = n - 1, n2 = n1 * n1;
   const unsigned qp = q > p, rp = r > p, rq = r > q;  // 1 where the first is the larger
   const unsigned cq = q - qp - (1u - rq), cp = p - (1u - qp) - (1u - rp);
-  // tile (a, la, b, lb) = ((a n + la) (n-1) + b') (n-1) + lb'; row c'', column
+  // tile (a, la, b, lb) = ((a n + la) (n-1) + b') (n-1) + lb'
   const unsigned ib = i * n * n2, jb = j * n * n2, kb = k * n * n2;
-  const unsigned t[6] = {ib + (j - 1) * n1 + p * n2 + (q - qp), ib + (k - 1) * n1 + p * n2 + (r - rp),
-                         jb + i * n1 + q * n2 + (p - (1u - qp)), jb + (k - 1) * n1 + q * n2 + (r - rq),
-                         kb + i * n1 + r * n2 + (p - (1u - rp)), kb + j * n1 + r * n2 + (q - (1u - rq))};
-  const unsigned row[6] = {(unsigned)k - 2, (unsigned)j - 1, (unsigned)k - 2, (unsigned)i, (unsigned)j - 1, (unsigned)i};
-  const unsigned col[6] = {(unsigned)cr, cq, (unsigned)cr, cp, cq, cp};
-  double D[6], w[6];
-  unsigned at[6];
+  ClassIdx x{{ib + (j - 1) * n1 + p * n2 + (q - qp), ib + (k - 1) * n1 + p * n2 + (r - rp),
+              jb + i * n1 + q * n2 + (p - (1u - qp)), jb + (k - 1) * n1 + q * n2 + (r - rq),
+              kb + i * n1 + r * n2 + (p - (1u - rp)), kb + j * n1 + r * n2 + (q - (1u - rq))},
+             {},
+             {(unsigned)k - 2, (unsigned)j - 1, (unsigned)k - 2, (unsigned)i, (unsigned)j - 1, (unsigned)i},
+             {(unsigned)cr, cq, (unsigned)cr, cp, cq, cp},
+             {},
+             {i * n + p, i * n + p, j * n + q, j * n + q, k * n + r, k * n + r}};
 #pragma unroll
   for (int b = 0; b < 6; ++b) {
-    const unsigned tm = RLT2_IDX(t[b], n * n * n2) * m;
-    at[b] = (tm + RLT2_IDX(row[b], m)) * m + RLT2_IDX(col[b], m);
-    D[b] = a.Dhat[at[b]];
-    w[b] = dadd_(ldv<RO>(a.xi + tm + row[b]), ldv<RO>(a.psi + tm + col[b]));
+    x.t[b] = RLT2_IDX(x.t[b], n * n * n2);
+    x.tm[b] = x.t[b] * m;
+    x.at[b] = (x.tm[b] + RLT2_IDX(x.row[b], m)) * m + RLT2_IDX(x.col[b], m);
+  }
+  return x;
+}
+
+// The folded move of a class in the integer form (FP64 where the exponents ask
+// for it).
+template <bool RO>
+__device__ __forceinline__ void move_class_fixed(const MoveZArgs& a, const ClassIdx& x) {
+  double D[6], w[6];
+#pragma unroll
+  for (int b = 0; b < 6; ++b) {
+    D[b] = a.Dhat[x.at[b]];
+    w[b] = dadd_(ldv<RO>(a.xi + x.tm[b] + x.row[b]), ldv<RO>(a.psi + x.tm[b] + x.col[b]));
   }
   if (!move_class_fx(D, w, a.phi_fx)) {
     double s[6], S = 0.0;
@@ -316,30 +264,115 @@ __device__ __forceinline__ void move_class_fixed(const MoveZArgs& a, int i, int 
     for (int b = 0; b < 6; ++b) D[b] = __fma_rn(a.c1, s[b], __fma_rn(a.w[0], S, D[b]));
   }
 #pragma unroll
-  for (int b = 0; b < 6; ++b) a.Dhat[at[b]] = D[b];
+  for (int b = 0; b < 6; ++b) a.Dhat[x.at[b]] = D[b];
 }
 
-// Work of the integer form's launches.  Each of a class's six planes (ordered
-// facility pair, third facility) is contiguous in one of the three locations
-// and a new row for every pair of the other two, so a warp's lanes cover 2 p x
-// 4 q x 4 r: 64 segments of two to four entries for its 192 (32 (q, r) of one p
-// take 144, a band of 8 q x 4 r 96).  The (q, r) of a p run in bands of eight
-// q, r outer, in groups of 32 slots (8 q x 4 r), so that only the last group
-// has idle lanes for any n; the four warps of a group hold its two q halves
-// for two pairs of p, and the two groups of a block the next four r, so that
-// the sectors that a segment shares with its neighbours are read once.
-__host__ __device__ inline int fixed_groups(int n) { return ((n - 1) * (n - 2) + 31) / 32; }
-__host__ __device__ inline int fixed_warps(int n) { return (n + 3) / 4 * fixed_groups(n) * 4; }  // per triple
+// The move of a class in FP64, in the oracle's operation order.
+template <bool RO>
+__device__ __forceinline__ void move_class_fp64(const MoveZArgs& a, const ClassIdx& x) {
+  RLT2_CLASS_TABLES
+  (void)kOrd;
+  // Half-Z scheme (Section 5): the upper members (i,j,k|p,q,r), (i,k,j|p,r,q) and
+  // (j,k,i|q,r,p) -- members 0, 1, 3 -- pool s = kz pi_z + tile term and each
+  // receives half of the other two pools: D' = D - s + (S - s)/2 with S the sum
+  // of the three pools in member order, evaluated as fma(-3/2, s, fma(1/2, S, D)).
+  // Lower members are never touched.
+  if (a.half) {
+    constexpr int kUp[3] = {0, 1, 3};
+    double s[3], Dv[3];
+#pragma unroll
+    for (int u = 0; u < 3; ++u) {
+      const int b = kUp[u];
+      Dv[u] = a.Dhat[x.at[b]];
+      const double pz = dsub_(dsub_(Dv[u], ldv<RO>(a.xi + x.tm[b] + x.row[b])), ldv<RO>(a.psi + x.tm[b] + x.col[b]));
+      const double ty = ldv<RO>(a.tterm + x.t[b]);
+      s[u] = a.kz_one ? dadd_(pz, ty) : __fma_rn(a.kz, pz, ty);
+    }
+    const double S = dadd_(dadd_(s[0], s[1]), s[2]);
+#pragma unroll
+    for (int u = 0; u < 3; ++u) a.Dhat[x.at[kUp[u]]] = __fma_rn(-1.5, s[u], __fma_rn(0.5, S, Dv[u]));
+    return;
+  }
+  double s[6], base[6];
+  if (a.folded) {
+    // the uniform pool of Eq. 2.20-2.23 with kz = 1, regrouped:
+    // D' = D - s + phi (S - s) = (D + phi S) - (1 + phi) s
+#pragma unroll
+    for (int b = 0; b < 6; ++b) {
+      base[b] = a.Dhat[x.at[b]];
+      s[b] = dsub_(dsub_(base[b], ldv<RO>(a.xi + x.tm[b] + x.row[b])), ldv<RO>(a.psi + x.tm[b] + x.col[b]));
+    }
+    double S = s[0];
+#pragma unroll
+    for (int b = 1; b < 6; ++b) S = dadd_(S, s[b]);
+#pragma unroll
+    for (int b = 0; b < 6; ++b) a.Dhat[x.at[b]] = __fma_rn(a.c1, s[b], __fma_rn(a.w[0], S, base[b]));
+    return;
+  }
+  const bool sa = a.fast && a.sc->sa_on;
+#pragma unroll
+  for (int b = 0; b < 6; ++b) {
+    const double Dv = a.Dhat[x.at[b]];
+    const double pz = dsub_(dsub_(Dv, ldv<RO>(a.xi + x.tm[b] + x.row[b])), ldv<RO>(a.psi + x.tm[b] + x.col[b]));
+    const double ty = ldv<RO>(a.tterm + x.t[b]);
+    // s = kz*pi_z + tile term in one rounding (kz = 1: an exact fma(1, x, y) is x + y)
+    s[b] = a.kz_one ? dadd_(pz, ty) : __fma_rn(a.kz, pz, ty);
+    if (!a.fast) {
+      base[b] = dsub_(Dv, s[b]);
+    } else {
+      // (1 - kz) pi_z in one rounding; fma(-1, x, x) is +0 exactly
+      base[b] = a.kz_one ? 0.0 : __fma_rn(-a.kz, pz, pz);
+      if (sa) base[b] = dsub_(base[b], ldv<RO>(a.saterm + x.fl[b]));
+    }
+  }
+  if (a.uniform) {
+    // all phi equal: member b receives phi * (S - s_b), S the class sum in member order
+    double S = s[0];
+#pragma unroll
+    for (int b = 1; b < 6; ++b) S = dadd_(S, s[b]);
+#pragma unroll
+    for (int b = 0; b < 6; ++b) a.Dhat[x.at[b]] = __fma_rn(a.w[0], dsub_(S, s[b]), base[b]);
+  } else {
+    // partner inflows one fused multiply-add at a time, partners in Eq. 2.20 order
+#pragma unroll
+    for (int b = 0; b < 6; ++b) {
+      double acc = base[b];
+#pragma unroll
+      for (int l = 0; l < 5; ++l) acc = __fma_rn(a.w[l], s[kPart[b][l]], acc);
+      a.Dhat[x.at[b]] = acc;
+    }
+  }
+}
 
-// Warp w (of fixed_warps) of triple tr.
-__device__ __forceinline__ void move_z_fixed_warp(const MoveZArgs& a, int tr, int w, int lane) {
-  const int n = a.n, m = a.m, n1 = n - 1;
-  const int quad = (int)__umulhi((unsigned)(w >> 2) << 1, a.rcp_groups);  // (w / 4) / fixed_groups
-  const int g = (w >> 2) - quad * fixed_groups(n);
+// Work of the moves' launches.  Each of a class's six planes (ordered facility
+// pair, third facility) is contiguous in one of the three locations and a new
+// row for every pair of the other two, so a warp's lanes cover 2 p x 4 q x 4 r:
+// 64 segments of two to four entries for its 192 (32 (q, r) of one p take 144, a
+// band of 8 q x 4 r 96).  The (q, r) of a p run in bands of eight q, r outer, in
+// groups of 32 slots (8 q x 4 r), so that only the last group has idle lanes for
+// any n; the four warps of a group hold its two q halves for two pairs of p, and
+// the two groups of a block the next four r, so that the sectors that a segment
+// shares with its neighbours are read once.
+__host__ __device__ inline int class_groups(int n) { return ((n - 1) * (n - 2) + 31) / 32; }
+__host__ __device__ inline int class_warps(int n) { return (n + 3) / 4 * class_groups(n) * 4; }  // per triple
+
+inline ClassRcp class_rcp(int n) {
+  auto rcp = [](unsigned d) { return (unsigned)(((1ull << 31) + d - 1) / d); };
+  return ClassRcp{rcp((unsigned)class_groups(n)), rcp(8u * (unsigned)(n - 2))};
+}
+
+// The class of lane `lane` of warp w (of class_warps) of triple tr, passed to
+// f(const ClassIdx&) if there is one.
+template <typename F>
+__device__ __forceinline__ void class_of_lane(int n, int m, const ClassRcp& rcp, const int* trips, int tr, int w,
+                                              int lane, F&& f) {
+  const int n1 = n - 1;
+  const int quad = (int)__umulhi((unsigned)(w >> 2) << 1, rcp.groups);  // (w / 4) / class_groups
+  const int g = (w >> 2) - quad * class_groups(n);
   const int p = 4 * quad + ((w & 1) << 1) + ((lane >> 2) & 1);
   const int u = 32 * g + ((lane & 3) << 3 | (w & 2) << 1 | lane >> 3);
   if (p >= n || u >= n1 * m) return;
-  const int band = (int)__umulhi((unsigned)u << 1, a.rcp_8m);  // u / (8 m)
+  const int band = (int)__umulhi((unsigned)u << 1, rcp.m8);  // u / (8 m)
   const int cb = u - band * 8 * m, hb = min(8, n1 - 8 * band);
   const int rr = hb == 8 ? cb >> 3 : cb / hb;
   const int qq = 8 * band + cb - rr * hb;
@@ -348,101 +381,35 @@ __device__ __forceinline__ void move_z_fixed_warp(const MoveZArgs& a, int tr, in
   int r = rr;
   r += (r >= lo);
   r += (r >= hi);
-  const int packed = a.trips[tr];
-  move_class_fixed<true>(a, packed & 255, (packed >> 8) & 255, packed >> 16, p, q, r, rr);
+  const int packed = trips[tr];
+  f(class_idx(n, m, packed & 255, (packed >> 8) & 255, packed >> 16, p, q, r, rr));
 }
 
-// The classes (q, r) = first, first + stride, ... of block blk = (triple, p);
-// BAND: the banded class order for n >= 22 (see class_of).  FIXED: the launch
-// may be asked for the integer form (a.fixed).
-template <bool RO = true, bool BAND = true, bool FIXED = false>
-__device__ __forceinline__ void move_z_block(const MoveZArgs& a, int blk, int first, int stride) {
-  if (a.half) {
-    move_z_half_block(a, blk);
-    return;
-  }
-  RLT2_CLASS_TABLES
-  const int n = a.n, m = a.m, n1 = n - 1;
-  const int tr = blk / n, p = blk - tr * n;
+// One class per lane of warp w of triple tr.
+template <bool FIXED>
+__device__ __forceinline__ void move_z_warp(const MoveZArgs& a, int tr, int w, int lane) {
+  class_of_lane(a.n, a.m, a.rcp, a.trips, tr, w, lane, [&](const ClassIdx& x) {
+    if constexpr (FIXED) move_class_fixed<true>(a, x);
+    else move_class_fp64<true>(a, x);
+  });
+}
+
+// The pipelined launch's unit: the classes (q, r) of block blk = (triple, p), one
+// warp, r fastest.  FIXED: the launch may be asked for the integer form.
+template <bool FIXED>
+__device__ __forceinline__ void move_z_block(const MoveZArgs& a, int blk, int lane) {
+  const int n = a.n, m = a.m, tr = blk / n, p = blk - tr * n;
   const int packed = a.trips[tr];
-  const int F3[3] = {packed & 255, (packed >> 8) & 255, packed >> 16};
-  const int npairs = n1 * m;
-  const long long mm = (long long)m * m;
-  const bool sa = a.fast && a.sc->sa_on;
-  for (int c = first; c < npairs; c += stride) {
-    int qq, rr;
-    class_of<BAND>(c, n1, m, qq, rr);
+  for (int c = lane; c < (n - 1) * m; c += 32) {
+    const int qq = c / m, rr = c - qq * m;
     const int q = qq + (qq >= p);
     const int lo = p < q ? p : q, hi = p < q ? q : p;
     int r = rr;
     r += (r >= lo);
     r += (r >= hi);
-    if (FIXED && a.fixed) {
-      move_class_fixed<RO>(a, F3[0], F3[1], F3[2], p, q, r, rr);
-      continue;
-    }
-    const int L3[3] = {p, q, r};
-    double s[6], base[6];
-    long long idx[6];
-    if (a.folded) {
-      // the uniform pool of Eq. 2.20-2.23 with kz = 1, regrouped:
-      // D' = D - s + phi (S - s) = (D + phi S) - (1 + phi) s
-      double Dv[6];
-#pragma unroll
-      for (int b = 0; b < 6; ++b) {
-        const int f0 = F3[kOrd[b][0]], f1 = F3[kOrd[b][1]], f2 = F3[kOrd[b][2]];
-        const int l0 = L3[kOrd[b][0]], l1 = L3[kOrd[b][1]], l2 = L3[kOrd[b][2]];
-        const long long t = RLT2_IDX(((long long)(f0 * n + l0) * n1 + (f1 - (f1 > f0))) * n1 + (l1 - (l1 > l0)),
-                                        (long long)n * n * n1 * n1);
-        const int kr = RLT2_IDX(f2 - (f2 > f0) - (f2 > f1), m), cc = RLT2_IDX(l2 - (l2 > l0) - (l2 > l1), m);
-        idx[b] = t * mm + kr * m + cc;
-        Dv[b] = a.Dhat[idx[b]];
-        s[b] = dsub_(dsub_(Dv[b], ldv<RO>(a.xi + t * m + kr)), ldv<RO>(a.psi + t * m + cc));
-      }
-      double S = s[0];
-#pragma unroll
-      for (int b = 1; b < 6; ++b) S = dadd_(S, s[b]);
-#pragma unroll
-      for (int b = 0; b < 6; ++b) a.Dhat[idx[b]] = __fma_rn(a.c1, s[b], __fma_rn(a.w[0], S, Dv[b]));
-      continue;
-    }
-#pragma unroll
-    for (int b = 0; b < 6; ++b) {
-      const int f0 = F3[kOrd[b][0]], f1 = F3[kOrd[b][1]], f2 = F3[kOrd[b][2]];
-      const int l0 = L3[kOrd[b][0]], l1 = L3[kOrd[b][1]], l2 = L3[kOrd[b][2]];
-      const long long t = RLT2_IDX(((long long)(f0 * n + l0) * n1 + (f1 - (f1 > f0))) * n1 + (l1 - (l1 > l0)),
-                                        (long long)n * n * n1 * n1);
-      const int kr = RLT2_IDX(f2 - (f2 > f0) - (f2 > f1), m), cc = RLT2_IDX(l2 - (l2 > l0) - (l2 > l1), m);
-      idx[b] = t * mm + kr * m + cc;
-      const double Dv = a.Dhat[idx[b]];
-      const double pz = dsub_(dsub_(Dv, ldv<RO>(a.xi + t * m + kr)), ldv<RO>(a.psi + t * m + cc));
-      // s = kz*pi_z + tile term in one rounding (kz = 1: an exact fma(1, x, y) is x + y)
-      s[b] = a.kz_one ? dadd_(pz, ldv<RO>(a.tterm + t)) : __fma_rn(a.kz, pz, ldv<RO>(a.tterm + t));
-      if (!a.fast) {
-        base[b] = dsub_(Dv, s[b]);
-      } else {
-        // (1 - kz) pi_z in one rounding; fma(-1, x, x) is +0 exactly
-        base[b] = a.kz_one ? 0.0 : __fma_rn(-a.kz, pz, pz);
-        if (sa) base[b] = dsub_(base[b], ldv<RO>(a.saterm + f0 * n + l0));
-      }
-    }
-    if (a.uniform) {
-      // all phi equal: member b receives phi * (S - s_b), S the class sum in member order
-      double S = s[0];
-#pragma unroll
-      for (int b = 1; b < 6; ++b) S = dadd_(S, s[b]);
-#pragma unroll
-      for (int b = 0; b < 6; ++b) a.Dhat[idx[b]] = __fma_rn(a.w[0], dsub_(S, s[b]), base[b]);
-    } else {
-      // partner inflows one fused multiply-add at a time, partners in Eq. 2.20 order
-#pragma unroll
-      for (int b = 0; b < 6; ++b) {
-        double acc = base[b];
-#pragma unroll
-        for (int l = 0; l < 5; ++l) acc = __fma_rn(a.w[l], s[kPart[b][l]], acc);
-        a.Dhat[idx[b]] = acc;
-      }
-    }
+    const ClassIdx x = class_idx(n, m, packed & 255, (packed >> 8) & 255, packed >> 16, p, q, r, rr);
+    if (FIXED && a.fixed) move_class_fixed<false>(a, x);
+    else move_class_fp64<false>(a, x);
   }
 }
 
@@ -453,6 +420,8 @@ __device__ __forceinline__ void move_z_block(const MoveZArgs& a, int blk, int fi
 struct Phase2Args {
   int n, m;
   double tol;
+  int tol_exp;  // exponent field of tol less 1023
+  ClassRcp rcp;
   double* Dhat;
   const double* xi;
   const double* psi;
@@ -460,56 +429,50 @@ struct Phase2Args {
   const DevScalars* sc;
 };
 
-__device__ __forceinline__ void phase2_block(const Phase2Args& a, int blk) {
-  RLT2_CLASS_TABLES
-  (void)kPart;
-  const int n = a.n, m = a.m, n1 = n - 1;
-  const int tr = blk / n, p = blk - tr * n;
-  const int packed = a.trips[tr];
-  const int F3[3] = {packed & 255, (packed >> 8) & 255, packed >> 16};
-  const int npairs = n1 * m;
-  const long long mm = (long long)m * m;
-  for (int c = threadIdx.x; c < npairs; c += blockDim.x) {
-    int qq, rr;
-    class_of(c, n1, m, qq, rr);
-    const int q = qq + (qq >= p);
-    const int lo = p < q ? p : q, hi = p < q ? q : p;
-    int r = rr;
-    r += (r >= lo);
-    r += (r >= hi);
-    const int L3[3] = {p, q, r};
-    double pz[6], Dv[6];
-    long long idx[6];
-    int nb = 0;
-    unsigned basic = 0;
-    double sum = 0.0;
-#pragma unroll
-    for (int b = 0; b < 6; ++b) {
-      const int f0 = F3[kOrd[b][0]], f1 = F3[kOrd[b][1]], f2 = F3[kOrd[b][2]];
-      const int l0 = L3[kOrd[b][0]], l1 = L3[kOrd[b][1]], l2 = L3[kOrd[b][2]];
-      const long long t = RLT2_IDX(((long long)(f0 * n + l0) * n1 + (f1 - (f1 > f0))) * n1 + (l1 - (l1 > l0)),
-                                        (long long)n * n * n1 * n1);
-      const int kr = RLT2_IDX(f2 - (f2 > f0) - (f2 > f1), m), cc = RLT2_IDX(l2 - (l2 > l0) - (l2 > l1), m);
-      idx[b] = t * mm + kr * m + cc;
-      Dv[b] = a.Dhat[idx[b]];
-      const double xv = __ldg(a.xi + t * m + kr), pv = __ldg(a.psi + t * m + cc);
-      pz[b] = dsub_(dsub_(Dv[b], xv), pv);
-      const double lim = dmul_(a.tol, dadd_(dadd_(1.0, fabs(xv)), fabs(pv)));
-      if (okey_(pz[b]) <= okey_(lim)) {
-        basic |= 1u << b;
-        ++nb;
-      } else {
-        sum = dadd_(sum, pz[b]);
-      }
-    }
-    if (nb == 0 || nb == 6) continue;
-    // 1/|S_B| as a correctly rounded constant, as in 1.0 / k
-    const double inv = nb == 1 ? 1.0 : nb == 2 ? 0.5 : nb == 3 ? 1.0 / 3.0 : nb == 4 ? 0.25 : 0.2;
-    const double share = dmul_(sum, inv);
-#pragma unroll
-    for (int b = 0; b < 6; ++b)
-      a.Dhat[idx[b]] = ((basic >> b) & 1u) ? dadd_(Dv[b], share) : dsub_(Dv[b], pz[b]);
+__device__ __forceinline__ int exp_field(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
+
+// pz <= tol (1 + |xv| + |pv|), the right side rounded sum by sum.  With E the
+// largest exponent field of 1, xv and pv and F = E + tol_exp, the right side is
+// at least 2^(F - 1023) (for a normal tol) and below 2^(F + 4 - 1023), so that
+// most slacks are decided by their exponent and the three FP64 operations are
+// needed for the few between.
+__device__ __forceinline__ bool in_basis(const Phase2Args& a, double pz, double xv, double pv) {
+  if (__double2hiint(pz) < 0) return true;  // negative or -0: the right side is >= 0
+  const int E = max(max(exp_field(xv), exp_field(pv)), 1023), F = E + a.tol_exp, e = exp_field(pz);
+  if (E < 2040) {
+    if (e >= F + 4) return false;
+    if (e < F - 1 && a.tol_exp > -1023) return true;
   }
+  return okey_(pz) <= okey_(dmul_(a.tol, dadd_(dadd_(1.0, fabs(xv)), fabs(pv))));
+}
+
+__device__ __forceinline__ void phase2_class(const Phase2Args& a, const ClassIdx& x) {
+  double pz[6], Dv[6];
+  int nb = 0;
+  unsigned basic = 0;
+  double sum = 0.0;
+#pragma unroll
+  for (int b = 0; b < 6; ++b) {
+    Dv[b] = a.Dhat[x.at[b]];
+    const double xv = __ldg(a.xi + x.tm[b] + x.row[b]), pv = __ldg(a.psi + x.tm[b] + x.col[b]);
+    pz[b] = dsub_(dsub_(Dv[b], xv), pv);
+    if (in_basis(a, pz[b], xv, pv)) {
+      basic |= 1u << b;
+      ++nb;
+    } else {
+      sum = dadd_(sum, pz[b]);
+    }
+  }
+  if (nb == 0 || nb == 6) return;
+  // 1/|S_B| as a correctly rounded constant, as in 1.0 / k
+  const double inv = nb == 1 ? 1.0 : nb == 2 ? 0.5 : nb == 3 ? 1.0 / 3.0 : nb == 4 ? 0.25 : 0.2;
+  const double share = dmul_(sum, inv);
+#pragma unroll
+  for (int b = 0; b < 6; ++b) a.Dhat[x.at[b]] = dadd_(Dv[b], ((basic >> b) & 1u) ? share : -pz[b]);
+}
+
+__device__ __forceinline__ void phase2_warp(const Phase2Args& a, int tr, int w, int lane) {
+  class_of_lane(a.n, a.m, a.rcp, a.trips, tr, w, lane, [&](const ClassIdx& x) { phase2_class(a, x); });
 }
 
 // ---------------------------------------------------------------- finalize ----
@@ -611,16 +574,6 @@ __device__ __forceinline__ void finalize_block(const FinArgs& a) {
       sc->reason = 3;
     }
   }
-}
-
-// Threads of a z-move block: the (n-1)(n-2) classes of one (triple, p) in
-// equal passes of at most 352 threads, rounded to whole warps (n = 20: one
-// pass of 352; three such blocks fit an SM at 62 registers, against two of
-// up to 512 threads: 4 % faster).
-inline int move_z_threads(int n) {
-  const int c = (n - 1) * (n - 2);
-  const int passes = (c + 351) / 352;
-  return ((c + passes - 1) / passes + 31) / 32 * 32;
 }
 
 // Kernel arguments of one problem's moves and finalize step (host helpers).
