@@ -531,7 +531,8 @@ struct rlt2_mlp {
   float *W1 = nullptr, *b1 = nullptr, *W2 = nullptr, *b2 = nullptr, *w3 = nullptr, *b3 = nullptr;
   bf16 *W1b = nullptr, *W2b = nullptr;
   float* mom = nullptr;  // 2 * nparams
-  float* grad = nullptr; // nparams, same packing as the parameters
+  float* grad = nullptr; // nparams, same packing as the parameters; loss and err behind it
+  char* host = nullptr;  // pinned copy of the same
   long long nparams = 0;
   int adam_t = 0;
   float gate = 0.0f;
@@ -547,6 +548,8 @@ struct rlt2_mlp {
 };
 
 namespace {
+size_t grad_bytes(const rlt2_mlp* m) { return ((size_t)m->nparams * sizeof(float) + 15) / 16 * 16 + 16; }
+
 // parameter packing: W1 [64 x H] | b1 [H] | W2 [H x H] | b2 [H] | w3 [H] | b3 [1]
 void param_ptrs(rlt2_mlp* m) {
   const int H = m->H;
@@ -742,7 +745,14 @@ extern "C" rlt2_status rlt2_mlp_create(int hidden, unsigned long long seed, void
   if ((e = cudaMalloc((void**)&m->W1, sizeof(float) * m->nparams)) != cudaSuccess) return fail(e);
   param_ptrs(m);
   if ((e = cudaMalloc((void**)&m->mom, sizeof(float) * 2 * m->nparams)) != cudaSuccess) return fail(e);
-  if ((e = cudaMalloc((void**)&m->grad, sizeof(float) * m->nparams)) != cudaSuccess) return fail(e);
+  // gradients, then the loss and the wait flag, so that one copy brings all three
+  if ((e = cudaMalloc((void**)&m->grad, grad_bytes(m))) != cudaSuccess) return fail(e);
+  m->loss = reinterpret_cast<double*>(reinterpret_cast<char*>(m->grad) + grad_bytes(m) - 16);
+  m->err = reinterpret_cast<int*>(m->loss + 1);
+  if (cudaMallocHost((void**)&m->host, grad_bytes(m)) != cudaSuccess) {
+    m->host = nullptr;  // rlt2_mlp_grad then copies into pageable memory
+    (void)cudaGetLastError();
+  }
   if ((e = cudaMalloc((void**)&m->W1b, sizeof(bf16) * kInPad * H)) != cudaSuccess) return fail(e);
   if ((e = cudaMalloc((void**)&m->W2b, sizeof(bf16) * H * H)) != cudaSuccess) return fail(e);
   const size_t cr = kChunk + 64;
@@ -754,8 +764,6 @@ extern "C" rlt2_status rlt2_mlp_create(int hidden, unsigned long long seed, void
   if ((e = cudaMalloc((void**)&m->out, sizeof(float) * cr)) != cudaSuccess) return fail(e);
   if ((e = cudaMalloc((void**)&m->tgt, sizeof(float) * cr)) != cudaSuccess) return fail(e);
   if ((e = cudaMalloc((void**)&m->scale, sizeof(float) * cr)) != cudaSuccess) return fail(e);
-  if ((e = cudaMalloc((void**)&m->loss, sizeof(double))) != cudaSuccess) return fail(e);
-  if ((e = cudaMalloc((void**)&m->err, sizeof(int))) != cudaSuccess) return fail(e);
   if ((e = cudaMemsetAsync(m->err, 0, sizeof(int), m->stream)) != cudaSuccess) return fail(e);
   cudaStream_t s = m->stream;
   // He initialisation of W1 (34 valid input rows) and W2, small w3, zero biases
@@ -774,9 +782,10 @@ extern "C" rlt2_status rlt2_mlp_destroy(rlt2_mlp* m) {
   if (!m) return RLT2_OK;
   if (m->stream) cudaStreamSynchronize(m->stream);
   void* ptrs[] = {m->W1, m->mom, m->grad, m->W1b, m->W2b, m->Xd, m->Td, m->Xc, m->H1, m->H2, m->dH1, m->dH2,
-                  m->out, m->tgt, m->scale, m->loss, m->err};
+                  m->out, m->tgt, m->scale};
   for (void* p : ptrs)
     if (p) cudaFree(p);
+  if (m->host) cudaFreeHost(m->host);
   delete m;
   return RLT2_OK;
 }
@@ -890,20 +899,27 @@ extern "C" rlt2_status rlt2_mlp_grad(rlt2_mlp* m, long long rows, double* loss, 
   const int H = m->H;
   cudaStream_t s = m->stream;
   const long long prows = (rows + 63) / 64 * 64;
-  CKM(cudaMemcpyAsync(m->Xc, m->Xd, sizeof(bf16) * rows * kInPad, cudaMemcpyDeviceToDevice, s));
-  if (prows > rows) CKM(cudaMemsetAsync(m->Xc + rows * kInPad, 0, sizeof(bf16) * (prows - rows) * kInPad, s));
-  CKM(cudaMemcpyAsync(m->tgt, m->Td, sizeof(float) * rows, cudaMemcpyDeviceToDevice, s));
-  CKM(cudaMemsetAsync(m->grad, 0, sizeof(float) * m->nparams, s));
-  CKM(cudaMemsetAsync(m->loss, 0, sizeof(double), s));
-  CKM(backward(m, m->Xc, m->tgt, prows, rows, s));
-  std::vector<float> g(m->nparams);
-  double l = 0.0;
-  CKM(cudaMemcpyAsync(g.data(), m->grad, sizeof(float) * m->nparams, cudaMemcpyDeviceToHost, s));
-  CKM(cudaMemcpyAsync(&l, m->loss, sizeof(double), cudaMemcpyDeviceToHost, s));
+  const bf16* X = m->Xd;
+  const float* T = m->Td;
+  if (prows > rows) {  // whole GEMM tiles: zero rows behind the samples
+    CKM(cudaMemcpyAsync(m->Xc, m->Xd, sizeof(bf16) * rows * kInPad, cudaMemcpyDeviceToDevice, s));
+    CKM(cudaMemsetAsync(m->Xc + rows * kInPad, 0, sizeof(bf16) * (prows - rows) * kInPad, s));
+    X = m->Xc;
+  }
+  const size_t bytes = grad_bytes(m);
+  CKM(cudaMemsetAsync(m->grad, 0, bytes - sizeof(double), s));  // gradients and loss
+  CKM(backward(m, X, T, prows, rows, s));
+  std::vector<char> pageable(m->host ? 0 : bytes);
+  char* g = m->host ? m->host : pageable.data();
+  CKM(cudaMemcpyAsync(g, m->grad, bytes, cudaMemcpyDeviceToHost, s));
   CKM(cudaStreamSynchronize(s));
-  if (rlt2_status ts = tc_wait_status(m, "rlt2_mlp_grad"); ts != RLT2_OK) return ts;
+  int waited = 0;
+  double l = 0.0;
+  memcpy(&l, g + bytes - 16, sizeof l);
+  memcpy(&waited, g + bytes - 8, sizeof waited);
+  if (waited) return tc_wait_status(m, "rlt2_mlp_grad");
   if (loss) *loss = l;
-  const float* p = g.data();
+  const float* p = reinterpret_cast<const float*>(g);
   if (gW1) memcpy(gW1, p, sizeof(float) * kIn * H);
   p += kInPad * H;
   if (gb1) memcpy(gb1, p, sizeof(float) * H);
