@@ -1,5 +1,6 @@
 // Batched LAP kernel (one warp per LAP) and the rlt2_lap_batched entry point.
 #include <cmath>
+#include <cstdint>
 #include <cstdio>
 #include <mutex>
 #include <type_traits>
@@ -119,7 +120,12 @@ __device__ __forceinline__ void k_lap_prefetching(const LapArgs& a, unsigned cha
     if (tb < a.batch) {
       const long long t = a.map ? (long long)a.map[tb] : tb;
       const double* src = a.A + t * mm;
-      for (int e = gl; e < mm; e += G) cp_async8(raw + e, src + e);
+      if (a.wide) {
+#pragma unroll 2
+        for (int e = 2 * gl; e < mm; e += 2 * G) cp_async16(raw + e, src + e);
+      } else {
+        for (int e = gl; e < mm; e += G) cp_async8(raw + e, src + e);
+      }
       if (warm && gl < m) cp_async8(raw + mm + gl, a.u0 + t * m + gl);
     }
     cp_async_commit();
@@ -138,6 +144,7 @@ __device__ __forceinline__ void k_lap_prefetching(const LapArgs& a, unsigned cha
     __syncwarp();
     unsigned eb = 0;
     if (have)
+#pragma unroll 4
       for (int e = gl; e < mm; e += G) eb = max(eb, fx_expfield_hi(raw + e));
     if constexpr (G == 32) {
       eb = __reduce_max_sync(kFull, eb);
@@ -467,6 +474,7 @@ cudaError_t launch_lap(const LapArgs& a, cudaStream_t s) {
   if (e != cudaSuccess) return e;
   LapArgs b = a;
   b.prefetch = plan.prefetch;
+  b.wide = !(a.m & 1) && (reinterpret_cast<std::uintptr_t>(a.A) & 15) == 0;
   const long long per_block = (long long)wpb * (32 / G);
   const long long need = (a.batch + per_block - 1) / per_block;
   const int grid = (int)(need < cap ? need : cap);

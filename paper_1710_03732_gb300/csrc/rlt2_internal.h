@@ -102,6 +102,7 @@ struct LapArgs {
                              // the next tile by cp.async while it solves the current one
   unsigned long long* head;  // nullable: device counter of the prefetching form's LAP queue
                              // (launch_lap zeroes it on the stream before the launch)
+  int wide;                  // set by launch_lap: tiles start on 16-byte boundaries (m even, A aligned)
   int dependent;             // launched as a programmatic dependent (see launch_dependent)
   int head_zeroed;           // an earlier launch on the stream has zeroed *head: no memset
 };

@@ -128,6 +128,11 @@ __device__ __forceinline__ void cp_async8(void* dst_smem, const void* src) {
   const unsigned sa = (unsigned)__cvta_generic_to_shared(dst_smem);
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(sa), "l"(src) : "memory");
 }
+// 16 bytes, both sides on a 16-byte boundary.
+__device__ __forceinline__ void cp_async16(void* dst_smem, const void* src) {
+  const unsigned sa = (unsigned)__cvta_generic_to_shared(dst_smem);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(src) : "memory");
+}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
 
@@ -473,8 +478,8 @@ __device__ __forceinline__ long long fx_floor_words(unsigned hi, unsigned lo, un
 // possibly the tile itself; the column reduction converts it into cs and then
 // calls hook().  kk = (L + 1075) << 20 for the tile's grid 2^L.
 // Bound by the ALU pipe (77 % busy) and issue (80 %).  Z stage, warm: n = 20 394
-// -> 370 us (3,160 -> 2,840 warp instructions per LAP: 580 the column
-// reduction, 950 the searches, 650 the canonical pass), n = 17 160 -> 139,
+// -> 356 us (3,160 -> 2,700 warp instructions per LAP: 580 the column
+// reduction, 900 the searches, 620 the canonical pass), n = 17 160 -> 139,
 // n = 12 41.5 -> 34.
 template <int G, bool RR = false, typename Hook = NoHook>
 __device__ __forceinline__ WarpLapResult<long long> group_lap_fx(long long* cs, int ld, int m, int lane, bool warm,
@@ -587,6 +592,15 @@ __device__ __forceinline__ WarpLapResult<long long> group_lap_fx(long long* cs, 
         }
       }
     }
+    if constexpr (G == 32) {
+      if (__ballot_sync(kFull, cv && kh == kOut) == 0) {  // the nearest column was free: no dual changes
+        if (gl == sink) {
+          c2r = i;
+          um = cs[i * ld + gl] - v;
+        }
+        continue;
+      }
+    }
     // the k-th scanned column relaxed the m - k columns still unscanned
     const bool scanned = act && cv && kh == kOut;
     const int step = __popc(group_bits<G>(__ballot_sync(kFull, scanned), gb));
@@ -654,6 +668,7 @@ __device__ __forceinline__ WarpLapResult<long long> group_lap_fx(long long* cs, 
   }
   int rs0 = 0;
   for (int it = 0; it < M - 1; ++it) {
+    if (it) rs0 = fx_argmin<G>(kh, (unsigned)dist, gb);
     const T es = __shfl_sync(kFull, dist - vown, gb + rs0);
     const int s = __shfl_sync(kFull, r2c, gb + rs0);
     if (G == 32 || it < m - 1) {
@@ -664,7 +679,6 @@ __device__ __forceinline__ WarpLapResult<long long> group_lap_fx(long long* cs, 
         kh = hi32(nd);
       }
     }
-    if (it + 2 < M) rs0 = fx_argmin<G>(kh, (unsigned)dist, gb);
   }
   const T u0r = __shfl_sync(kFull, u, gb);
   const T ucan = cv ? dist + (u - u0r) : T(0);
