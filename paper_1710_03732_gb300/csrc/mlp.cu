@@ -35,7 +35,12 @@ namespace {
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kIn = 34;      // features per row
 constexpr int kInPad = 64;   // padded input width (GEMM K)
-constexpr int kChunk = 1 << 18;  // rows per inference/training chunk
+constexpr int kChunk = 1 << 18;  // rows per training chunk, and per inference chunk of widths other than 256
+// Rows per inference chunk of the 256-wide network (features, predictions and
+// scales only): 64 MB of features, which stay in L2.  At m = 18 a chunk is three
+// full waves of feature warps and 27 of the network's tiles, where 2^18 rows were
+// one and a half and 13.5: 144,400 tiles 1.10 -> 0.96 ms.
+constexpr int kPredictChunk = 1 << 19;
 using bf16 = __nv_bfloat16;
 
 // x with its significand cut to FP32: the exponent field less 896 (its low eight
@@ -50,20 +55,46 @@ __device__ __forceinline__ float f32_trunc(double x) {
 }
 
 // ------------------------------------------------------------- features ----
-// Ascending bitonic sort of `width` lanes (8, 16 or 32; the lanes past a row's
+// Ascending bitonic sort of W lanes (8, 16 or 32; the lanes past a row's
 // end hold the largest key) of two rows at once: unsigned 16-bit keys, row i in
-// the low half.
-__device__ __forceinline__ unsigned sort_rows(unsigned v, int width, int lane) {
+// the low half.  A lane that keeps the larger key of a pair works on the
+// complement, where that is the smaller one; its partner is on the other side,
+// so a stage is one shuffle, x = min(x, ~o) and the change of sides to the next
+// stage: bit of flip[stage] per lane, all ones or zero.
+struct SortFlips {
+  unsigned f[16];  // f[0] before the first stage, f[s] after stage s
+};
+template <int W>
+__device__ __forceinline__ SortFlips sort_flips(int lane) {
+  SortFlips x{};
+  unsigned side = 0;
+  int s = 0;
 #pragma unroll
   for (int k = 2; k <= 32; k <<= 1) {
-    if (k > width) break;
+    if (k <= W) {
 #pragma unroll
-    for (int j = k >> 1; j > 0; j >>= 1) {
-      const unsigned o = __shfl_xor_sync(kFull, v, j);
-      v = ((lane & j) == 0) == ((lane & k) == 0) ? __vminu2(v, o) : __vmaxu2(v, o);
+      for (int j = k >> 1; j > 0; j >>= 1) {
+        const unsigned now = ((lane & j) == 0) != ((lane & k) == 0) ? ~0u : 0u;
+        x.f[s++] = side ^ now;
+        side = now;
+      }
+      x.f[s] = side;  // back to plain keys if this was the last stage
     }
   }
-  return v;
+  return x;
+}
+template <int W>
+__device__ __forceinline__ unsigned sort_rows(unsigned v, const SortFlips& x) {
+  int s = 0;
+#pragma unroll
+  for (int k = 2; k <= W; k <<= 1) {
+#pragma unroll
+    for (int j = k >> 1; j > 0; j >>= 1) {
+      v ^= x.f[s++];
+      v = __vminu2(v, ~__shfl_xor_sync(kFull, v, j));
+    }
+  }
+  return v ^ x.f[s];
 }
 // The same on floats, one row (scaled rows that overflow FP32).
 __device__ __forceinline__ float sort_row(float v, int lane) {
@@ -88,6 +119,7 @@ __device__ __forceinline__ float sort_row(float v, int lane) {
 // 144,400 tiles of size 18: 72 -> 43 us per 262,144 rows, the whole prediction
 // 1.41 -> 1.11 ms.
 constexpr int kFeatWarps = 8;
+template <int W>
 __global__ void __launch_bounds__(kFeatWarps * 32) k_features(long long ntiles, int m,
                                                               const double* __restrict__ tiles,
                                                               const double* __restrict__ prev_u,
@@ -98,7 +130,7 @@ __global__ void __launch_bounds__(kFeatWarps * 32) k_features(long long ntiles, 
   const int lane = threadIdx.x & 31;
   const bool col = lane < m;
   float* sm = feat_smem + (threadIdx.x >> 5) * m * m;
-  const int width = m <= 8 ? 8 : m <= 16 ? 16 : 32;
+  const SortFlips flips = sort_flips<W>(lane);
   const unsigned mword = (unsigned)__bfloat16_as_ushort(__float2bfloat16_rn((float)m / 32.0f)) << 16;
   const long long nw = (long long)gridDim.x * (blockDim.x >> 5);
   for (long long t = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); t < ntiles; t += nw) {
@@ -129,7 +161,7 @@ __global__ void __launch_bounds__(kFeatWarps * 32) k_features(long long ntiles, 
       unsigned w;
       if (s <= 3.402823466e38f) {
         const __nv_bfloat162 r = __floats2bfloat162_rn(va, vb);
-        w = sort_rows(*reinterpret_cast<const unsigned*>(&r), width, lane);
+        w = sort_rows<W>(*reinterpret_cast<const unsigned*>(&r), flips);
       } else {
         const __nv_bfloat162 r = __floats2bfloat162_rn(sort_row(va, lane), sort_row(vb, lane));
         w = *reinterpret_cast<const unsigned*>(&r);
@@ -152,10 +184,14 @@ __global__ void __launch_bounds__(kFeatWarps * 32) k_features(long long ntiles, 
     }
   }
 }
-static int feat_grid(long long ntiles) {
-  return (int)std::min<long long>(8192, (ntiles + kFeatWarps - 1) / kFeatWarps);
+static cudaError_t launch_features(long long ntiles, int m, const double* tiles, const double* prev_u,
+                                   const double* target_u, bf16* X, float* target, float* scale, cudaStream_t s) {
+  const auto kern = m <= 8 ? k_features<8> : m <= 16 ? k_features<16> : k_features<32>;
+  const int grid = (int)std::min<long long>(8192, (ntiles + kFeatWarps - 1) / kFeatWarps);
+  kern<<<grid, kFeatWarps * 32, (size_t)kFeatWarps * m * m * sizeof(float), s>>>(ntiles, m, tiles, prev_u, target_u, X,
+                                                                               target, scale);
+  return cudaGetLastError();
 }
-static size_t feat_smem_bytes(int m) { return (size_t)kFeatWarps * m * m * sizeof(float); }
 
 // ----------------------------------------------------------------- GEMM ----
 // C[M x N] = A[M x K] * B[K x N] with BF16 inputs and FP32 accumulation on the
@@ -695,13 +731,13 @@ cudaError_t umma_mlp_forward(const bf16* X, long long rows, const bf16* W1, cons
 cudaError_t mlp_predict_enqueue(rlt2_mlp* m, long long ntiles, int mz, const double* tiles, const double* prev_u,
                                 double* u0, cudaStream_t s, int* launched) {
   cudaError_t e;
-  const long long tiles_per_chunk = std::max<long long>(1, kChunk / mz);
+  const long long tiles_per_chunk = std::max<long long>(1, (m->H == 256 ? kPredictChunk : kChunk) / mz);
   for (long long t0 = 0; t0 < ntiles; t0 += tiles_per_chunk) {
     const long long nt = std::min(tiles_per_chunk, ntiles - t0);
     const long long rows = nt * mz, prows = (rows + 63) / 64 * 64;
-    k_features<<<feat_grid(nt), kFeatWarps * 32, feat_smem_bytes(mz), s>>>(
-        nt, mz, tiles + t0 * mz * mz, prev_u ? prev_u + t0 * mz : nullptr, nullptr, m->Xc, nullptr, m->scale);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = launch_features(nt, mz, tiles + t0 * mz * mz, prev_u ? prev_u + t0 * mz : nullptr, nullptr, m->Xc, nullptr,
+                             m->scale, s)) != cudaSuccess)
+      return e;
     if (prows > rows && (e = cudaMemsetAsync(m->Xc + rows * kInPad, 0, sizeof(bf16) * (prows - rows) * kInPad, s)) !=
                             cudaSuccess)
       return e;
@@ -757,15 +793,15 @@ extern "C" rlt2_status rlt2_mlp_create(int hidden, unsigned long long seed, void
   }
   if ((e = cudaMalloc((void**)&m->W1b, sizeof(bf16) * kInPad * H)) != cudaSuccess) return fail(e);
   if ((e = cudaMalloc((void**)&m->W2b, sizeof(bf16) * H * H)) != cudaSuccess) return fail(e);
-  const size_t cr = kChunk + 64;
-  if ((e = cudaMalloc((void**)&m->Xc, sizeof(bf16) * cr * kInPad)) != cudaSuccess) return fail(e);
+  const size_t cr = kChunk + 64, pr = kPredictChunk + 64;
+  if ((e = cudaMalloc((void**)&m->Xc, sizeof(bf16) * pr * kInPad)) != cudaSuccess) return fail(e);
   if ((e = cudaMalloc((void**)&m->H1, sizeof(bf16) * cr * H)) != cudaSuccess) return fail(e);
   if ((e = cudaMalloc((void**)&m->H2, sizeof(bf16) * cr * H)) != cudaSuccess) return fail(e);
   if ((e = cudaMalloc((void**)&m->dH1, sizeof(bf16) * cr * H)) != cudaSuccess) return fail(e);
   if ((e = cudaMalloc((void**)&m->dH2, sizeof(bf16) * cr * H)) != cudaSuccess) return fail(e);
-  if ((e = cudaMalloc((void**)&m->out, sizeof(float) * cr)) != cudaSuccess) return fail(e);
+  if ((e = cudaMalloc((void**)&m->out, sizeof(float) * pr)) != cudaSuccess) return fail(e);
   if ((e = cudaMalloc((void**)&m->tgt, sizeof(float) * cr)) != cudaSuccess) return fail(e);
-  if ((e = cudaMalloc((void**)&m->scale, sizeof(float) * cr)) != cudaSuccess) return fail(e);
+  if ((e = cudaMalloc((void**)&m->scale, sizeof(float) * pr)) != cudaSuccess) return fail(e);
   if ((e = cudaMemsetAsync(m->err, 0, sizeof(int), m->stream)) != cudaSuccess) return fail(e);
   cudaStream_t s = m->stream;
   // He initialisation of W1 (34 valid input rows) and W2, small w3, zero biases
@@ -851,9 +887,8 @@ extern "C" rlt2_status rlt2_mlp_add_samples(rlt2_mlp* m, long long ntiles, int m
   CKM(ensure_dataset(m, m->rows + ntiles * mz));
   float* scale = nullptr;
   CKM(cudaMalloc((void**)&scale, sizeof(float) * ntiles));
-  k_features<<<feat_grid(ntiles), kFeatWarps * 32, feat_smem_bytes(mz), m->stream>>>(
-      ntiles, mz, tiles, prev_u, target_u, m->Xd + m->rows * kInPad, m->Td + m->rows, scale);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch_features(ntiles, mz, tiles, prev_u, target_u, m->Xd + m->rows * kInPad, m->Td + m->rows, scale,
+                                  m->stream);
   cudaError_t e2 = cudaStreamSynchronize(m->stream);
   cudaFree(scale);
   if (e != cudaSuccess) return cuda_fail(e, "k_features");
