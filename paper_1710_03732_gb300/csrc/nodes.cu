@@ -5,7 +5,7 @@
 // admitted into waves that fit a device-memory budget, each node gets its own
 // arena (D^, C^, duals, scalars) carved from one pool, and every stage of an
 // iteration runs as one launch over all nodes of the wave:
-//   k_move_y_nodes / k_move_z_nodes  grid.y = node
+//   k_move_y_nodes / k_move_z_nodes  blockIdx.y = node
 //   k_lap_nodes (Z, Y, X)            persistent warps pulling LAPs of all nodes
 //                                    from a device queue (lap.cu)
 //   k_finalize_nodes                 one block per node
@@ -38,22 +38,26 @@ __global__ void k_move_y_nodes(const MoveYArgs* nodes) {
   else move_y_range(a, start, stride);
 }
 
-// blockIdx.y = triple, blockIdx.z = node, eight of the triple's warps per block.
+// blockIdx.x = triple, blockIdx.y = node; a block goes through the triple's warps,
+// so that the node's arguments, read from global memory, cost one latency per
+// triple and nodes smaller than the largest leave few empty blocks (64 nodes of
+// residual 14 to 18: 350 -> 341 ms for 20 iterations against a block per eight
+// warps).
 template <bool FIXED>
 __global__ void __launch_bounds__(256, 4) k_move_z_nodes(const MoveZArgs* nodes, const int* ntrips) {
-  const MoveZArgs& a = nodes[blockIdx.z];
-  const int w = blockIdx.x * 8 + (threadIdx.x >> 5);
-  if ((int)blockIdx.y >= ntrips[blockIdx.z] || w >= class_warps(a.n)) return;
+  const MoveZArgs& a = nodes[blockIdx.y];
+  if ((int)blockIdx.x >= ntrips[blockIdx.y]) return;
   if (!a.sc->have_snap || a.sc->done) return;
-  move_z_warp<FIXED>(a, blockIdx.y, w, threadIdx.x & 31);
+#pragma unroll 1
+  for (int w = threadIdx.x >> 5; w < class_warps(a.n); w += 8)
+    move_z_warp<FIXED>(a, blockIdx.x, w, threadIdx.x & 31, false);
 }
 
 __global__ void __launch_bounds__(256, 4) k_phase2_nodes(const Phase2Args* nodes, const int* ntrips) {
-  const Phase2Args& a = nodes[blockIdx.z];
-  const int w = blockIdx.x * 8 + (threadIdx.x >> 5);
-  if ((int)blockIdx.y >= ntrips[blockIdx.z] || w >= class_warps(a.n)) return;
-  if (a.sc->done) return;
-  phase2_warp(a, blockIdx.y, w, threadIdx.x & 31);
+  const Phase2Args& a = nodes[blockIdx.y];
+  if ((int)blockIdx.x >= ntrips[blockIdx.y] || a.sc->done) return;
+#pragma unroll 1
+  for (int w = threadIdx.x >> 5; w < class_warps(a.n); w += 8) phase2_warp(a, blockIdx.x, w, threadIdx.x & 31);
 }
 
 __global__ void __launch_bounds__(256) k_finalize_nodes(const FinArgs* nodes) {
@@ -249,7 +253,7 @@ cudaError_t enqueue_wave_iteration(const Wave& w, const WaveDev& d, int dual_mod
     k_move_y_nodes<<<dim3(bx, w.nn), 256, 0, s>>>(d.my);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
-  const dim3 class_grid((class_warps(w.max_n) + 7) / 8, w.max_trips, w.nn);
+  const dim3 class_grid(w.max_trips, w.nn);
   if (w.fixed) k_move_z_nodes<true><<<class_grid, 256, 0, s>>>(d.mz, d.mz_trips);
   else k_move_z_nodes<false><<<class_grid, 256, 0, s>>>(d.mz, d.mz_trips);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
