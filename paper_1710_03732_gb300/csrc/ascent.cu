@@ -117,17 +117,15 @@ __global__ void k_move_y(MoveYArgs a) {
 // the folded move.  Four blocks per SM at 64 registers.  Integer form: 0.291 ms at
 // n = 20 (two to five blocks 0.309, 0.309, 0.293), 3.72 ms at n = 30, against
 // 0.461 and 6.3 ms for the FP64 form; bound by the L2 tags (73 % busy, a request
-// per segment), then the FP64 pipe (54 %) and the ALU pipe (42 %); the stop flags
-// are looked at before the stores, so that their load does not precede the
-// class's (288 -> 285 us); blocks of 4 or 16 warps and several groups per warp
-// are slower (288, 308, 331 us).  FP64 form:
+// per segment), then the FP64 pipe (54 %) and the ALU pipe (42 %); blocks of 4 or
+// 16 warps and several groups per warp are slower (291, 310, 331 us).  FP64 form:
 // n = 20 folded 461 -> 454 us with these lanes, n = 16 126 -> 120.
 template <bool FIXED>
 __global__ void __launch_bounds__(256, 4) k_move_z(MoveZArgs a) {
   dependent_begin();
-  const bool stopped = !a.sc->have_snap || a.sc->done;
+  if (!a.sc->have_snap || a.sc->done) return;
   const int w = blockIdx.x * 8 + (threadIdx.x >> 5);
-  if (w < class_warps(a.n)) move_z_warp<FIXED>(a, blockIdx.y, w, threadIdx.x & 31, stopped);
+  if (w < class_warps(a.n)) move_z_warp<FIXED>(a, blockIdx.y, w, threadIdx.x & 31);
 }
 
 // Second phase of the two-phase Z solve; runs on every iteration (the first

@@ -50,7 +50,7 @@ __global__ void __launch_bounds__(256, 4) k_move_z_nodes(const MoveZArgs* nodes,
   if (!a.sc->have_snap || a.sc->done) return;
 #pragma unroll 1
   for (int w = threadIdx.x >> 5; w < class_warps(a.n); w += 8)
-    move_z_warp<FIXED>(a, blockIdx.x, w, threadIdx.x & 31, false);
+    move_z_warp<FIXED>(a, blockIdx.x, w, threadIdx.x & 31);
 }
 
 __global__ void __launch_bounds__(256, 4) k_phase2_nodes(const Phase2Args* nodes, const int* ntrips) {

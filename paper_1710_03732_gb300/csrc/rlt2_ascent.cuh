@@ -246,7 +246,7 @@ __device__ __forceinline__ ClassIdx class_idx(unsigned n, unsigned m, int i, int
 // The folded move of a class in the integer form (FP64 where the exponents ask
 // for it).
 template <bool RO>
-__device__ __forceinline__ void move_class_fixed(const MoveZArgs& a, const ClassIdx& x, bool stopped) {
+__device__ __forceinline__ void move_class_fixed(const MoveZArgs& a, const ClassIdx& x) {
   double D[6], w[6];
 #pragma unroll
   for (int b = 0; b < 6; ++b) {
@@ -263,7 +263,6 @@ __device__ __forceinline__ void move_class_fixed(const MoveZArgs& a, const Class
 #pragma unroll
     for (int b = 0; b < 6; ++b) D[b] = __fma_rn(a.c1, s[b], __fma_rn(a.w[0], S, D[b]));
   }
-  if (stopped) return;
 #pragma unroll
   for (int b = 0; b < 6; ++b) a.Dhat[x.at[b]] = D[b];
 }
@@ -386,12 +385,11 @@ __device__ __forceinline__ void class_of_lane(int n, int m, const ClassRcp& rcp,
   f(class_idx(n, m, packed & 255, (packed >> 8) & 255, packed >> 16, p, q, r, rr));
 }
 
-// One class per lane of warp w of triple tr.  stopped: nothing may be stored.
+// One class per lane of warp w of triple tr.
 template <bool FIXED>
-__device__ __forceinline__ void move_z_warp(const MoveZArgs& a, int tr, int w, int lane, bool stopped) {
-  if (!FIXED && stopped) return;
+__device__ __forceinline__ void move_z_warp(const MoveZArgs& a, int tr, int w, int lane) {
   class_of_lane(a.n, a.m, a.rcp, a.trips, tr, w, lane, [&](const ClassIdx& x) {
-    if constexpr (FIXED) move_class_fixed<true>(a, x, stopped);
+    if constexpr (FIXED) move_class_fixed<true>(a, x);
     else move_class_fp64<true>(a, x);
   });
 }
@@ -410,7 +408,7 @@ __device__ __forceinline__ void move_z_block(const MoveZArgs& a, int blk, int la
     r += (r >= lo);
     r += (r >= hi);
     const ClassIdx x = class_idx(n, m, packed & 255, (packed >> 8) & 255, packed >> 16, p, q, r, rr);
-    if (FIXED && a.fixed) move_class_fixed<false>(a, x, false);
+    if (FIXED && a.fixed) move_class_fixed<false>(a, x);
     else move_class_fp64<false>(a, x);
   }
 }
