@@ -74,14 +74,21 @@ __device__ __forceinline__ void k_lap_one_tile(const LapArgs& a, unsigned char* 
     const int L = fx_grid(eb);
     const T u0 = (warm && lane < m) ? start_dual<true>(u0d, L) : T(0);
     long long next = a.batch;
-    const WarpLapResult<T> R = group_lap_fx<G, RR>(tile, ld, m, lane, warm, u0, scr, uv, raw, ld, L, [&]() {
+    auto advance = [&]() {
       t_static += stride;
       next = claim_step<1>(a, t_static, lane);
       if (next < a.batch) {
         const char* p = reinterpret_cast<const char*>(a.A + slot(next) * mm);
         for (int o = lane * 128; o < mm * 8; o += 32 * 128) asm volatile("prefetch.global.L2 [%0];" ::"l"(p + o));
       }
-    });
+    };
+    WarpLapResult<T> R;
+    if (!warm && eb == 0 && group_all_zero<32>(raw, m * ld, lane, 1)) {
+      zero_tile_result(R, lane, m);
+      advance();
+    } else {
+      R = group_lap_fx<G, RR>(tile, ld, m, lane, warm, u0, scr, uv, raw, ld, L, advance);
+    }
     if (lane < m) {
       if (a.u) a.u[ts * m + lane] = out_value<true>(R.u, L);
       if (a.v) a.v[ts * m + lane] = out_value<true>(R.v, L);
@@ -156,12 +163,24 @@ __device__ __forceinline__ void k_lap_prefetching(const LapArgs& a, unsigned cha
     T u0 = T(0);
     if (warm && have && gl < m) u0 = start_dual<true>(raw[mm + gl], L);
     long long next = a.batch;  // claimed in the hook, which group_lap_fx calls once (raw is set)
-    const WarpLapResult<T> R = group_lap_fx<G, RR>(tile, ld, have ? m : 0, lane, warm, u0, scr, uv + grp * G, raw, m,
-                                                   L, [&]() {
-                                                     t_static += stride;
-                                                     next = claim(t_static);
-                                                     issue(next);
-                                                   });
+    auto advance = [&]() {
+      t_static += stride;
+      next = claim(t_static);
+      issue(next);
+    };
+    bool zero = false;  // this group's tile, from a cold start
+    if (!warm && __any_sync(kFull, have && eb == 0)) {
+      const bool all = group_all_zero<G>(raw, have ? mm : 0, gl, 1);
+      zero = have && all;
+    }
+    WarpLapResult<T> R;
+    if (__any_sync(kFull, have && !zero)) {
+      R = group_lap_fx<G, RR>(tile, ld, have && !zero ? m : 0, lane, warm, u0, scr, uv + grp * G, raw, m, L, advance);
+    } else {
+      __syncwarp();  // every lane's reads of raw are done
+      advance();
+    }
+    if (zero) zero_tile_result(R, gl, m);
     if (have && gl < m) {
       if (a.u) a.u[t * m + gl] = out_value<true>(R.u, L);
       if (a.v) a.v[t * m + gl] = out_value<true>(R.v, L);
@@ -226,8 +245,16 @@ __global__ void __launch_bounds__(kMaxWarpsPerBlock * 32, kLapBlocks<G>) k_lap(L
       stage_tile<G, false>(tile, ld, m, gl, have ? a.A + t * mm : nullptr, nullptr);
       const double u0 = (warm && have && gl < m) ? a.u0[t * m + gl] : 0.0;
       __syncwarp();
-      const WarpLapResult<double> R =
-          group_lap<G, true>(tile, ld, have ? m : 0, lane, warm, u0, a.dual_mode, scr, uv + grp * G);
+      bool zero = false;  // +0 throughout, cold: a glance at the first row's start, then all of the tile
+      if (!warm && __all_sync(kFull, !have || gl >= m || __double_as_longlong(tile[gl]) == 0)) {
+        bool all = true;  // rows are ld apart: one at a time
+        for (int r = 0; r < m; ++r) all = group_all_zero<G>(tile + r * ld, have ? m : 0, gl, 0) && all;
+        zero = have && all;
+      }
+      WarpLapResult<double> R;
+      if (__any_sync(kFull, have && !zero))
+        R = group_lap<G, true>(tile, ld, have && !zero ? m : 0, lane, warm, u0, a.dual_mode, scr, uv + grp * G);
+      if (zero) zero_tile_result(R, gl, m);
       if (have && gl < m) {
         if (a.u) a.u[t * m + gl] = R.u;
         if (a.v) a.v[t * m + gl] = R.v;
@@ -583,8 +610,20 @@ __device__ __forceinline__ void k_lap_nodes_prefetching(const NodeLapArgs& a, co
     }
     const int L = fx_grid(eb);
     const T u0 = (cur.warm && gl < m) ? start_dual<true>(raw[mm + gl], L) : T(0);
-    const WarpLapResult<T> R = group_lap_fx<G, RR>(tile, tile_ld(m), m, lane, cur.warm, u0, scr, uv + grp * G, raw, m,
-                                                   L, [&]() { issue(nxt); });
+    bool zero = false;  // this group's tile, from a cold start
+    if (__any_sync(kFull, cur.have && !cur.warm && eb == 0)) {
+      const bool all = group_all_zero<G>(raw, mm, gl, 1);
+      zero = cur.have && !cur.warm && all;
+    }
+    WarpLapResult<T> R;
+    if (__any_sync(kFull, cur.have && !zero)) {
+      R = group_lap_fx<G, RR>(tile, tile_ld(m), zero ? 0 : m, lane, cur.warm, u0, scr, uv + grp * G, raw, m, L,
+                              [&]() { issue(nxt); });
+    } else {
+      __syncwarp();  // every lane's reads of raw are done
+      issue(nxt);
+    }
+    if (zero) zero_tile_result(R, gl, m);
     if (cur.have) {
       const NodeLapItem& it = a.items[cur.k];
       if (gl < m) {

@@ -695,6 +695,35 @@ __device__ __forceinline__ WarpLapResult<long long> group_lap_fx(long long* cs, 
   return R;
 }
 
+// ---- all-zero tiles ------------------------------------------------------------
+// The first solve of every ascent has D^ = 0 (Algorithm 1, step 1): each tile is
+// zero, every argmin a tie, and the searches walk through all matched columns
+// (n = 30: 15.3 ms for that Z stage against 3.3 for a later one).  From a cold
+// start the outcome is known: column 0 takes row 0; the search of row i scans
+// columns 0 .. i-1 in lane order and takes column i; all duals stay 0.
+template <int G>
+__device__ __forceinline__ bool group_all_zero(const double* p, int count, int gl, unsigned ignore_sign) {
+  unsigned nz = 0;
+  for (int e = gl; e < count; e += G) {
+    const unsigned* w = reinterpret_cast<const unsigned*>(p + e);
+    nz |= w[0] | (w[1] << ignore_sign);
+  }
+  if constexpr (G == 32) {
+    nz = __reduce_or_sync(kFull, nz);
+  } else {
+#pragma unroll
+    for (int off = G / 2; off > 0; off >>= 1) nz |= __shfl_xor_sync(kFull, nz, off);
+  }
+  return nz == 0;
+}
+template <typename T>
+__device__ __forceinline__ void zero_tile_result(WarpLapResult<T>& R, int gl, int m) {
+  R.u = R.v = R.value = T(0);
+  R.r2c = R.c2r = gl;
+  R.naug = m - 1;
+  R.nrelax = m * (m - 1) + m * m * (m - 1) / 2 - (m - 1) * m * (m + 1) / 6;  // sum over i of m + i m - i (i+1) / 2
+}
+
 // ---- launch helpers shared by the LAP kernels ------------------------------
 constexpr int kMaxWarpsPerBlock = 8;
 
