@@ -64,7 +64,7 @@ def measured_peaks():
 # until one of them changes)
 KERNEL_SOURCES = {
     "lap_z": ["lap.cu", "rlt2_lap.cuh", "rlt2_internal.h"],
-    "move_z": ["rlt2_ascent.cuh", "rlt2_internal.h"],
+    "move_z": ["rlt2_ascent.cuh", "rlt2_internal.h", "rlt2_movefx.cuh"],
 }
 
 
@@ -763,8 +763,9 @@ def main():
     avg_lz64, fl_lz64, ach_lz64 = lap_z_roofline(f64)
     mz_ms = warm["kt"]["move_z"][0] / max(warm["kt"]["move_z"][1], 1)
     E = T * m * m
-    # folded uniform z move (kz = 1, equal phi): per entry 2 for s = (D - xi) - psi',
-    # 5/6 for the class sum S, 2 fused multiply-adds for D' = fma(-(1+phi), s, fma(phi, S, D))
+    # folded uniform z move (kz = 1, equal phi): in FP64 an entry would take 2 for
+    # s = (D - xi) - psi', 5/6 for the class sum S and 2 fused multiply-adds for
+    # D' = fma(-(1+phi), s, fma(phi, S, D)); dual_mode 1 sums its classes in integers
     mz_ops = E * (4 + 5.0 / 6.0)
     mz_bytes = E * 16 + 2 * T * m * 8  # D^ read + write, xi and psi' read once
     peaks = measured_peaks()
@@ -785,8 +786,9 @@ def main():
         "scaling": "weak",
         "vs_baseline": None,
         "dtype": "f64+i64",
-        "dtype_note": "FP64 state and multiplier moves (bit-exact with the oracle's operation order); "
-                      "LAPs in exact 64-bit fixed point on a per-tile grid of 2^-48 of the tile's magnitude",
+        "dtype_note": "FP64 state; z move summed in 64-bit integers on a grid per class (2^-6 of the FP64 rounding "
+                      "unit of its largest input), the other moves in FP64; LAPs in exact 64-bit fixed point on a "
+                      "per-tile grid of 2^-48 of the tile's magnitude",
         "data": "synthetic",
         "config": {"workload": WORKLOAD, "n": n, "z_laps_per_iter": T, "z_lap_size": m, "z_entries": E,
                    "warm_start": "previous-iteration Z duals", "parallelism": f"replicas x{world}",
@@ -819,7 +821,7 @@ def main():
                                     "(rlt2_probe_rates, CUDA events); nominal 64 lanes/clk/SM x 152 x 2.07 GHz = "
                                     f"{INT64_PEAK_GOPS:.0f}",
                      "limiter": "the ALU pipe's compares, selects and warp reductions of the sequential "
-                                "Dijkstra steps and instruction issue (ncu: ALU pipe 78 %, issue 81 % busy), "
+                                "Dijkstra steps and instruction issue (ncu: ALU pipe 77 %, issue 80 % busy), "
                                 "not the additions",
                      # the same additions counted as FP64 ops against the FP64 pipe (the roofline of
                      # an FP64 solve): above 1 means faster than an FP64 solve could be
@@ -834,15 +836,17 @@ def main():
                            "roofline_lap_z": {"bound": "alu", "achieved": ach_lz64, "peak": rates["dadd"],
                                               "unit": FP64_UNIT, "frac": ach_lz64 / rates["dadd"],
                                               "peak_source": "measured add.rn.f64 lane throughput"}},
-        "roofline_move_z": {"bound": "alu", "kernel": "move_z", "achieved": mz_ops / (mz_ms * 1e-3) / 1e9,
-                            "peak": fp64_move_peak, "unit": FP64_UNIT,
-                            "frac": mz_ops / (mz_ms * 1e-3) / 1e9 / fp64_move_peak, "traffic": traffic_mz,
-                            "algorithmic_ops_per_launch": mz_ops,
-                            "peak_source": "measured in this run: the kernel's FP64 mix (2 5/6 add/sub, 2 fma per "
-                                           "entry) at the probed add.rn.f64 and fma.rn.f64 lane rates",
-                            "frac_of_nominal": mz_ops / (mz_ms * 1e-3) / 1e9 / FP64_PEAK_GOPS,
-                            "hbm_gbs": mz_bytes / (mz_ms * 1e-3) / 1e9,
-                            "hbm_frac_of_measured": (mz_bytes / (mz_ms * 1e-3) / 1e9 / hbm) if hbm else None,
+        "roofline_move_z": {"bound": "hbm", "kernel": "move_z", "achieved": mz_bytes / (mz_ms * 1e-3) / 1e9,
+                            "peak": hbm, "unit": "GB/s",
+                            "frac": (mz_bytes / (mz_ms * 1e-3) / 1e9 / hbm) if hbm else None, "traffic": traffic_mz,
+                            "algorithmic_bytes_per_launch": mz_bytes,
+                            "arithmetic": "64-bit integers on one grid per class (dual_mode 1)",
+                            "peak_source": "MEASURED_PEAKS.json (copy bandwidth)",
+                            "limiter": "L2 tags: a request per two to four entries of a class's six planes (ncu: "
+                                       "73 % busy), then the FP64 pipe's conversions (54 %) and the ALU pipe (42 %)",
+                            # against the FP64 operations of the FP64 form at their measured rates:
+                            # above 1 means faster than that form could be
+                            "frac_of_fp64_form_peak": mz_ops / (mz_ms * 1e-3) / 1e9 / fp64_move_peak,
                             "avg_launch_ms": mz_ms},
         "cpu_baseline": cpu,
         "cpu_oracle_detail": cpu_detail,
