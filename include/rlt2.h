@@ -62,7 +62,10 @@ typedef enum {
  *               optimal row duals with u_0 = 0; unique for a given cost
  *               matrix) computed exactly in 64-bit fixed point on a per-tile
  *               grid of 2^-48 of the tile's magnitude bound, so warm and cold
- *               solves agree bit for bit, 2 = canonical duals computed in FP64
+ *               solves agree bit for bit (the z move of kz = 1 and equal phi_z
+ *               is then summed in 64-bit integers on a grid per class, at least
+ *               as close to the exact move as FP64), 2 = canonical duals
+ *               computed in FP64
  *  warm       : 0 = cold LAPs, 1 = start every Z, Y and X LAP from its
  *               previous iteration's row duals, 2 = as 1 but the Z-LAPs start
  *               from row duals predicted by the network attached with
@@ -337,8 +340,9 @@ long long rlt2_debug_bounds_violations(void);
  *  n_aug    : device, batch augmenting searches per LAP (nullable)
  *  dual_mode: 0 raw (FP64), 1 canonical (exact fixed point), 2 canonical
  *             (FP64), as in rlt2_params.  Asynchronous on `stream`; dual_mode
- *             1 takes 8 bytes of stream-ordered device memory for its work
- *             queue (cudaMallocAsync, freed on `stream` after the launch). */
+ *             1 takes 8 bytes of stream-ordered device memory for the work
+ *             queue of a batch that the resident warps do not hold at once
+ *             (freed on `stream` after the launch). */
 rlt2_status rlt2_lap_batched(int batch, int m, const double* cost, const double* u0, double* value, double* u,
                              double* v, int* row_to_col, int* n_aug, int dual_mode, void* stream);
 
