@@ -10,13 +10,14 @@
 //                equal phi) also psi <- psi - tile term, and it zeroes the Z
 //                stage's LAP queue counter
 //   k_move_z     class-owned z move (Eq. 2.20 + 2.22 + 2.23, combined as in the
-//                proof of Theorem 1), in place on D^ (Section 3.3)
+//                proof of Theorem 1), in place on D^ (Section 3.3); the folded
+//                form of canonical ascents in integers (rlt2_movefx.cuh)
 //   k_lap(Z)     n^2 (n-1)^2 LAPs of size n-2 on the tiles of D^ (half of them
 //                with the half-Z scheme, Section 5)
 //   [k_phase2, k_lap(Z)]  the two-phase Z solve (Section 3.4)
-//   k_lap(Y)     n^2 LAPs of size n-1 on C^ + Theta (fold fused into the tile
+//   k_lap_block(Y)  n^2 LAPs of size n-1 on C^ + Theta (fold fused into the tile
 //                load), writes pi_y
-//   k_lap(X)     one LAP of size n on b' + Delta, writes pi_x
+//   k_lap_block(X)  one LAP of size n on b' + Delta, writes pi_x
 //   k_finalize   bound, best bound, upper bound of the X primal, the feasibility
 //                check that follows Algorithm 1, stop flags, bound history
 // A context's first 64 iterations are launched kernel by kernel, later ones as

@@ -43,10 +43,11 @@ namespace rlt2 {
 constexpr int kPipeSpinLimit = 1 << 22;
 // The same limit in the failure-detection check, whose waits can never end.
 constexpr int kPipeCheckSpinLimit = 1 << 12;
-// Warps per block that run the move first (of kMaxWarpsPerBlock): 12 per SM
-// keep the FP64 pipe busy through the move's load latencies, the other 20 run
-// the integer LAPs (n = 20: 1, 2, 3, 4 tried, 3 fastest).
-constexpr int kMoveWarps = 3;
+// Warps per block that run the move first (of kMaxWarpsPerBlock): 8 per SM keep
+// the integer move going through its load latencies, the other 24 run the
+// integer LAPs (n = 20 cold, warm per iteration: two 1.36, 1.08 ms, three 1.47,
+// 1.14, four 1.46, 1.12).
+constexpr int kMoveWarps = 2;
 
 // 64 registers: four blocks of eight warps per SM (80 unbounded: three)
 template <int G, bool FX, bool RR = false>
