@@ -200,16 +200,6 @@ struct MoveZArgs {
   const DevScalars* sc;
 };
 
-// Loads of the duals and tile terms: through the read-only cache in the
-// stand-alone move; plain loads where the same launch later rewrites the duals
-// (the pipelined move + Z-LAP kernel, whose move reads of a tile's duals all
-// precede that tile's LAP).
-template <bool RO>
-__device__ __forceinline__ double ldv(const double* p) {
-  if constexpr (RO) return __ldg(p);
-  else return *p;
-}
-
 // Where the members of the class {(i,p),(j,q),(k,r)}, i < j < k, lie: member b's
 // entry at[b] of D^, its row dual xi[tm[b] + row[b]], column dual psi[tm[b] +
 // col[b]], tile t[b] and (first facility, first location) fl[b].  Member order as
@@ -245,13 +235,12 @@ __device__ __forceinline__ ClassIdx class_idx(unsigned n, unsigned m, int i, int
 
 // The folded move of a class in the integer form (FP64 where the exponents ask
 // for it).
-template <bool RO>
 __device__ __forceinline__ void move_class_fixed(const MoveZArgs& a, const ClassIdx& x) {
   double D[6], w[6];
 #pragma unroll
   for (int b = 0; b < 6; ++b) {
     D[b] = a.Dhat[x.at[b]];
-    w[b] = dadd_(ldv<RO>(a.xi + x.tm[b] + x.row[b]), ldv<RO>(a.psi + x.tm[b] + x.col[b]));
+    w[b] = dadd_(a.xi[x.tm[b] + x.row[b]], a.psi[x.tm[b] + x.col[b]]);
   }
   if (!move_class_fx(D, w, a.phi_fx)) {
     double s[6], S = 0.0;
@@ -268,7 +257,6 @@ __device__ __forceinline__ void move_class_fixed(const MoveZArgs& a, const Class
 }
 
 // The move of a class in FP64, in the oracle's operation order.
-template <bool RO>
 __device__ __forceinline__ void move_class_fp64(const MoveZArgs& a, const ClassIdx& x) {
   RLT2_CLASS_TABLES
   (void)kOrd;
@@ -284,8 +272,8 @@ __device__ __forceinline__ void move_class_fp64(const MoveZArgs& a, const ClassI
     for (int u = 0; u < 3; ++u) {
       const int b = kUp[u];
       Dv[u] = a.Dhat[x.at[b]];
-      const double pz = dsub_(dsub_(Dv[u], ldv<RO>(a.xi + x.tm[b] + x.row[b])), ldv<RO>(a.psi + x.tm[b] + x.col[b]));
-      const double ty = ldv<RO>(a.tterm + x.t[b]);
+      const double pz = dsub_(dsub_(Dv[u], a.xi[x.tm[b] + x.row[b]]), a.psi[x.tm[b] + x.col[b]]);
+      const double ty = a.tterm[x.t[b]];
       s[u] = a.kz_one ? dadd_(pz, ty) : __fma_rn(a.kz, pz, ty);
     }
     const double S = dadd_(dadd_(s[0], s[1]), s[2]);
@@ -300,7 +288,7 @@ __device__ __forceinline__ void move_class_fp64(const MoveZArgs& a, const ClassI
 #pragma unroll
     for (int b = 0; b < 6; ++b) {
       base[b] = a.Dhat[x.at[b]];
-      s[b] = dsub_(dsub_(base[b], ldv<RO>(a.xi + x.tm[b] + x.row[b])), ldv<RO>(a.psi + x.tm[b] + x.col[b]));
+      s[b] = dsub_(dsub_(base[b], a.xi[x.tm[b] + x.row[b]]), a.psi[x.tm[b] + x.col[b]]);
     }
     double S = s[0];
 #pragma unroll
@@ -313,8 +301,8 @@ __device__ __forceinline__ void move_class_fp64(const MoveZArgs& a, const ClassI
 #pragma unroll
   for (int b = 0; b < 6; ++b) {
     const double Dv = a.Dhat[x.at[b]];
-    const double pz = dsub_(dsub_(Dv, ldv<RO>(a.xi + x.tm[b] + x.row[b])), ldv<RO>(a.psi + x.tm[b] + x.col[b]));
-    const double ty = ldv<RO>(a.tterm + x.t[b]);
+    const double pz = dsub_(dsub_(Dv, a.xi[x.tm[b] + x.row[b]]), a.psi[x.tm[b] + x.col[b]]);
+    const double ty = a.tterm[x.t[b]];
     // s = kz*pi_z + tile term in one rounding (kz = 1: an exact fma(1, x, y) is x + y)
     s[b] = a.kz_one ? dadd_(pz, ty) : __fma_rn(a.kz, pz, ty);
     if (!a.fast) {
@@ -322,7 +310,7 @@ __device__ __forceinline__ void move_class_fp64(const MoveZArgs& a, const ClassI
     } else {
       // (1 - kz) pi_z in one rounding; fma(-1, x, x) is +0 exactly
       base[b] = a.kz_one ? 0.0 : __fma_rn(-a.kz, pz, pz);
-      if (sa) base[b] = dsub_(base[b], ldv<RO>(a.saterm + x.fl[b]));
+      if (sa) base[b] = dsub_(base[b], a.saterm[x.fl[b]]);
     }
   }
   if (a.uniform) {
@@ -389,8 +377,8 @@ __device__ __forceinline__ void class_of_lane(int n, int m, const ClassRcp& rcp,
 template <bool FIXED>
 __device__ __forceinline__ void move_z_warp(const MoveZArgs& a, int tr, int w, int lane) {
   class_of_lane(a.n, a.m, a.rcp, a.trips, tr, w, lane, [&](const ClassIdx& x) {
-    if constexpr (FIXED) move_class_fixed<true>(a, x);
-    else move_class_fp64<true>(a, x);
+    if constexpr (FIXED) move_class_fixed(a, x);
+    else move_class_fp64(a, x);
   });
 }
 
@@ -408,8 +396,8 @@ __device__ __forceinline__ void move_z_block(const MoveZArgs& a, int blk, int la
     r += (r >= lo);
     r += (r >= hi);
     const ClassIdx x = class_idx(n, m, packed & 255, (packed >> 8) & 255, packed >> 16, p, q, r, rr);
-    if (FIXED && a.fixed) move_class_fixed<false>(a, x);
-    else move_class_fp64<false>(a, x);
+    if (FIXED && a.fixed) move_class_fixed(a, x);
+    else move_class_fp64(a, x);
   }
 }
 
@@ -454,7 +442,7 @@ __device__ __forceinline__ void phase2_class(const Phase2Args& a, const ClassIdx
 #pragma unroll
   for (int b = 0; b < 6; ++b) {
     Dv[b] = a.Dhat[x.at[b]];
-    const double xv = __ldg(a.xi + x.tm[b] + x.row[b]), pv = __ldg(a.psi + x.tm[b] + x.col[b]);
+    const double xv = a.xi[x.tm[b] + x.row[b]], pv = a.psi[x.tm[b] + x.col[b]];
     pz[b] = dsub_(dsub_(Dv[b], xv), pv);
     if (in_basis(a, pz[b], xv, pv)) {
       basic |= 1u << b;

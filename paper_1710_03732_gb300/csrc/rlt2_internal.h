@@ -47,7 +47,12 @@ unsigned long long oob_fused();
 // running; dependent_begin() lets its own successor start in the same way and
 // then waits until everything before it has finished and is visible.  Called
 // first thing by every thread, before any global memory is touched, it leaves
-// the order that the stream gives; what overlaps is the launch itself.  In an
+// the order that the stream gives; what overlaps is the launch itself.  What the
+// wait makes visible is what ordinary (coherent) loads see: such a kernel may be
+// resident while its inputs are still written, so it reads nothing that an
+// earlier launch writes through the read-only path (__ldg, ld.global.nc, const
+// __restrict__ kernel parameters), whose data has to stay unwritten for as long
+// as the kernel lives.  In an
 // iteration the z move, the Y and X stages and k_finalize are launched this way
 // (kernel by kernel n = 8 45 -> 38 us per iteration, n = 12 78 -> 71, n = 20
 // 704 -> 697; in graph replay, whose gaps are short already, 31.3 and 31.0,
