@@ -42,11 +42,12 @@ __global__ void k_move_y_nodes(const MoveYArgs* nodes) {
 // so that the node's arguments, read from global memory, cost one latency per
 // triple and nodes smaller than the largest leave few empty blocks (64 nodes of
 // residual 14 to 18: 350 -> 341 ms for 20 iterations against a block per eight
-// warps).
+// warps).  FIXED: the nodes whose own parameters give the integer form, else the
+// others; a node moves as it would alone, whatever shares its wave.
 template <bool FIXED>
 __global__ void __launch_bounds__(256, 4) k_move_z_nodes(const MoveZArgs* nodes, const int* ntrips) {
   const MoveZArgs& a = nodes[blockIdx.y];
-  if ((int)blockIdx.x >= ntrips[blockIdx.y]) return;
+  if ((int)blockIdx.x >= ntrips[blockIdx.y] || (a.fixed != 0) != FIXED) return;
   if (!a.sc->have_snap || a.sc->done) return;
 #pragma unroll 1
   for (int w = threadIdx.x >> 5; w < class_warps(a.n); w += 8)
@@ -174,7 +175,7 @@ struct Wave {
   std::vector<LearnedStart> learned;  // one per node when warm == 2
   int nn = 0;
   int two_phase = 0;
-  int fixed = 1;  // every node's z move takes the integer form
+  bool moves[2] = {false, false};  // nodes whose z move takes the FP64 form, the integer form
   int cold = 0;  // warm == 0: no LAP of the wave has start duals
   long long total[kStages] = {0, 0, 0, 0};
   int max_m[kStages] = {0, 0, 0, 0};
@@ -254,8 +255,8 @@ cudaError_t enqueue_wave_iteration(const Wave& w, const WaveDev& d, int dual_mod
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   const dim3 class_grid(w.max_trips, w.nn);
-  if (w.fixed) k_move_z_nodes<true><<<class_grid, 256, 0, s>>>(d.mz, d.mz_trips);
-  else k_move_z_nodes<false><<<class_grid, 256, 0, s>>>(d.mz, d.mz_trips);
+  if (w.moves[1]) k_move_z_nodes<true><<<class_grid, 256, 0, s>>>(d.mz, d.mz_trips);
+  if (w.moves[0]) k_move_z_nodes<false><<<class_grid, 256, 0, s>>>(d.mz, d.mz_trips);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   for (const LearnedStart& ls : w.learned)
     if ((e = mlp_predict_enqueue(w.mlp, ls.T, ls.m, ls.Dhat, ls.xi, ls.u0, s)) != cudaSuccess) return e;
@@ -369,7 +370,7 @@ void add_node(Wave& w, WaveHost& h, int j, const IterView& v, const rlt2_params&
   }
   h.my[j] = make_move_y(v);
   h.mz[j] = make_move_z(v);
-  w.fixed = w.fixed && h.mz[j].fixed;
+  w.moves[h.mz[j].fixed] = true;
   h.p2[j] = make_phase2(v);
   h.mzb[j] = v.ntrip;
   h.fin[j] = make_fin(v);
