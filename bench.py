@@ -786,8 +786,8 @@ def main():
         "scaling": "weak",
         "vs_baseline": None,
         "dtype": "f64+i64",
-        "dtype_note": "FP64 state; z move summed in 64-bit integers on a grid per class (2^-6 of the FP64 rounding "
-                      "unit of its largest input), the other moves in FP64; LAPs in exact 64-bit fixed point on a "
+        "dtype_note": "FP64 state and moves, the slacks of a z class summed in 64-bit integers on a grid per class "
+                      "(at most 2^-58 of its largest slack); LAPs in exact 64-bit fixed point on a "
                       "per-tile grid of 2^-48 of the tile's magnitude",
         "data": "synthetic",
         "config": {"workload": WORKLOAD, "n": n, "z_laps_per_iter": T, "z_lap_size": m, "z_entries": E,
@@ -840,10 +840,10 @@ def main():
                             "peak": hbm, "unit": "GB/s",
                             "frac": (mz_bytes / (mz_ms * 1e-3) / 1e9 / hbm) if hbm else None, "traffic": traffic_mz,
                             "algorithmic_bytes_per_launch": mz_bytes,
-                            "arithmetic": "64-bit integers on one grid per class (dual_mode 1)",
+                            "arithmetic": "slacks in FP64, summed in 64-bit integers on one grid per class (dual_mode 1)",
                             "peak_source": "MEASURED_PEAKS.json (copy bandwidth)",
-                            "limiter": "L2 tags: a request per two to four entries of a class's six planes (ncu: "
-                                       "73 % busy), then the FP64 pipe's conversions (54 %) and the ALU pipe (42 %)",
+                            "limiter": "the FP64 pipe's slacks and additions (ncu: 79 % busy), then the L2 tags: a "
+                                       "request per two to four entries of a class's six planes (69 %)",
                             # against the FP64 operations of the FP64 form at their measured rates:
                             # above 1 means faster than that form could be
                             "frac_of_fp64_form_peak": mz_ops / (mz_ms * 1e-3) / 1e9 / fp64_move_peak,

@@ -63,9 +63,10 @@ typedef enum {
  *               matrix) computed exactly in 64-bit fixed point on a per-tile
  *               grid of 2^-48 of the tile's magnitude bound, so warm and cold
  *               solves agree bit for bit (the z move of kz = 1 and equal phi_z
- *               is then summed in 64-bit integers on a grid per class, at least
- *               as close to the exact move as FP64), 2 = canonical duals
- *               computed in FP64
+ *               then sums its slacks, formed in FP64, in 64-bit integers on a
+ *               grid per class: its root mean square error is no larger than
+ *               the FP64 form's, single entries may differ either way),
+ *               2 = canonical duals computed in FP64
  *  warm       : 0 = cold LAPs, 1 = start every Z, Y and X LAP from its
  *               previous iteration's row duals, 2 = as 1 but the Z-LAPs start
  *               from row duals predicted by the network attached with

@@ -115,12 +115,13 @@ __global__ void k_move_y(MoveYArgs a) {
 }
 
 // blockIdx.y = triple, eight of its warps per block; FIXED: the integer form of
-// the folded move.  Four blocks per SM at 64 registers.  Integer form: 0.291 ms at
-// n = 20 (two to five blocks 0.309, 0.309, 0.293), 3.72 ms at n = 30, against
-// 0.461 and 6.3 ms for the FP64 form; bound by the L2 tags (73 % busy, a request
-// per segment), then the FP64 pipe (54 %) and the ALU pipe (42 %); blocks of 4 or
-// 16 warps and several groups per warp are slower (291, 310, 331 us).  FP64 form:
-// n = 20 folded 461 -> 454 us with these lanes, n = 16 126 -> 120.
+// the folded move.  Four blocks per SM at 64 registers.  Integer form: 0.299 ms at
+// n = 20, 3.86 ms at n = 30, against 0.453 and 6.3 ms for the FP64 form; bound by
+// the FP64 pipe (79 % busy, 18 operations a class instead of 29), then the L2 tags
+// (69 %, a request per segment) and the ALU pipe (37 %).  Forming the slacks in
+// integers too takes 0.290 and 3.73 ms, but holds the smaller members of a class in
+// fewer bits than FP64 does.  FP64 form: n = 20 folded 461 -> 453 us with these
+// lanes, n = 16 126 -> 120.
 template <bool FIXED>
 __global__ void __launch_bounds__(256, 4) k_move_z(MoveZArgs a) {
   dependent_begin();

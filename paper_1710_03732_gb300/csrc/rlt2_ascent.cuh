@@ -188,7 +188,7 @@ struct MoveZArgs {
   int folded;   // S, kz = 1, all phi equal: psi holds psi - tile term, s = (D - xi) - psi,
                 // D' = fma(c1, s, fma(phi, S, D)) with c1 = -(1 + phi)
   double c1;
-  int fixed;        // folded move in integers (canonical duals in fixed point; see rlt2_movefx.cuh)
+  int fixed;        // folded move, slacks summed in integers (canonical duals in fixed point; see rlt2_movefx.cuh)
   FxFactor phi_fx;  // phi of the fixed form
   ClassRcp rcp;
   const double* saterm;  // n*n Type 4 amounts (F variant, when sc->sa_on)
@@ -233,22 +233,19 @@ __device__ __forceinline__ ClassIdx class_idx(unsigned n, unsigned m, int i, int
   return x;
 }
 
-// The folded move of a class in the integer form (FP64 where the exponents ask
-// for it).
+// The folded move of a class, its slacks summed in integers (FP64 where the
+// exponents ask for it).
 __device__ __forceinline__ void move_class_fixed(const MoveZArgs& a, const ClassIdx& x) {
-  double D[6], w[6];
+  double D[6], s[6];
 #pragma unroll
   for (int b = 0; b < 6; ++b) {
     D[b] = a.Dhat[x.at[b]];
-    w[b] = dadd_(a.xi[x.tm[b] + x.row[b]], a.psi[x.tm[b] + x.col[b]]);
+    s[b] = dsub_(dsub_(D[b], a.xi[x.tm[b] + x.row[b]]), a.psi[x.tm[b] + x.col[b]]);
   }
-  if (!move_class_fx(D, w, a.phi_fx)) {
-    double s[6], S = 0.0;
+  if (!pool_class_fx(D, s, a.phi_fx)) {
+    double S = s[0];
 #pragma unroll
-    for (int b = 0; b < 6; ++b) {
-      s[b] = dsub_(D[b], w[b]);
-      S = b ? dadd_(S, s[b]) : s[0];
-    }
+    for (int b = 1; b < 6; ++b) S = dadd_(S, s[b]);
 #pragma unroll
     for (int b = 0; b < 6; ++b) D[b] = __fma_rn(a.c1, s[b], __fma_rn(a.w[0], S, D[b]));
   }

@@ -1,26 +1,28 @@
-// The folded z move of one symmetry class in 64-bit integers (host and device).
+// The folded z move of one symmetry class with its pool in 64-bit integers (host
+// and device).
 //
-//   w_b  = xi_b + psi_b          b = 0..5, psi already less the tile term
-//   s_b  = D_b - w_b,  S = s_0 + ... + s_5
-//   D'_b = D_b - s_b + phi (S - s_b) = w_b + phi (S - s_b)
+//   s_b  = (D_b - xi_b) - psi_b     b = 0..5, psi already less the tile term
+//   S    = s_0 + ... + s_5
+//   D'_b = D_b + (phi (S - s_b) - s_b)
 //
 // GB300 retires FP64 operations at about 1.7 lanes per clock per SM and 32-bit
-// integer operations at about 128, so the 29 FP64 operations of a class cost
-// more than these sums in integers on one grid per class.  w_b is one FP64
-// addition (the FP64 pipe has room for six, and six integer conversions are
-// saved); D_b and w_b are cut onto the grid 2^L, L = emax - 1081 in biased
-// exponents, emax the largest exponent field among the class's D_b and w_b:
-//   - an input is |x| < 2^59 steps; those within 2^6 of the largest are exact,
-//     smaller ones are cut toward zero by less than one step;
-//   - |s_b| < 2^60, |S| < 2^62.6, |D'_b| < 2^61 (phi = 1/5): no overflow, and
-//     the sums are exact;
+// integer operations at about 128.  Of the FP64 form's 29 operations a class, the
+// twelve that form the s_b and six that add to the D_b stay in FP64: no input or
+// result is held in fewer bits than there, however far apart the members'
+// magnitudes are.  What lies between is summed on one grid per class, 2^L with
+// L = emax - 1081 in biased exponents, emax the largest exponent field of the s_b:
+//   - |s_b| < 2^59 steps; those within 2^6 of the largest are exact, smaller ones
+//     are cut toward zero by less than one step, 2^-59 to 2^-58 of the largest,
+//     where the FP64 form rounds every partial sum at up to 2^-53 of it;
+//   - |S| < 2^61.6, |phi (S - s_b) - s_b| < 2^60 (phi = 1/5): no overflow, and the
+//     sums are exact;
 //   - phi (S - s_b) is cut by less than three steps (see fx_scale);
-//   - D'_b is rounded once, to nearest, when it is stored as a double.
-// A step is 2^-6 of the rounding unit (2^-53) of the class's largest input,
-// where the FP64 form rounds two differences per entry and every sum at up to
-// that unit, so the result is at least as close to the exact move
-// (tests/test_movefx.py).  Exponents at the ends of the range, and infinities
-// or NaN, take the FP64 form.
+//   - the change of D_b is rounded once to a double, and D_b + change once.
+// The root mean square error against the exact move is no larger than the FP64
+// form's, over a class and member by member, also for classes with members 10^9
+// apart; a single entry can lie further off than there by a rounding unit of its
+// change (tests/test_movefx_pool.py compares both).  Exponents at the ends of the
+// range, infinities and NaN take the FP64 form.
 #pragma once
 #include <cstdint>
 #include <cstring>
@@ -76,15 +78,22 @@ RLT2_HD int64_t fx_align(double x, uint32_t emax) {
   return ((int64_t)q ^ neg) - neg;
 }
 
-// q grid steps as a double (rounded to nearest).
+// q grid steps as a double, rounded to nearest (ties away from zero), |q| < 2^62.
+// Integer operations only: a conversion instruction would cost the FP64 pipe as
+// much as an addition.
 RLT2_HD double fx_unalign(int64_t q, uint32_t emax) {
+  const uint64_t neg = (uint64_t)(q >> 63);
+  const uint64_t a = ((uint64_t)q ^ neg) - neg;
 #if defined(__CUDA_ARCH__)
-  const uint64_t b = fx_bits(__ll2double_rn(q));
+  const uint32_t z = (uint32_t)__clzll((long long)a);
 #else
-  const uint64_t b = fx_bits((double)q);
+  const uint32_t z = a ? (uint32_t)__builtin_clzll(a) : 64u;
 #endif
-  const uint32_t hi = (uint32_t)(b >> 32);  // 0 only for q = 0
-  return fx_double(((uint64_t)(hi ? hi + (emax - (1081u << 20)) : 0u) << 32) | (uint32_t)b);
+  // the leading bit at bit 62, half a unit added, then the unit at bit 0: a carry
+  // out of the significand raises the exponent
+  const uint64_t r = ((a << ((z - 1) & 63u)) + 0x200) >> 10;
+  const uint32_t e = emax + ((4u - z) << 20);  // less one: the leading bit, at bit 52 of r, adds it
+  return fx_double(a ? (((uint64_t)e << 32) + r) | (neg << 63) : 0);
 }
 
 // phi as hi 2^-32 + lo 2^-64 with lo signed, and phi x within three steps.
@@ -102,23 +111,50 @@ RLT2_HD int64_t fx_scale(FxFactor f, int64_t x) {
   return (int64_t)xh * f.hi + (int64_t)(((uint64_t)xl * (uint32_t)f.hi) >> 32) + (((int64_t)xh * f.lo) >> 32);
 }
 
-// The move of one class, in place on D, w_b = xi_b + psi_b; false (D untouched)
-// where the class's exponents call for the FP64 form.
-RLT2_HD bool move_class_fx(double D[6], const double w[6], FxFactor phi) {
-  uint32_t emax = 0;
+// The pool of one class on its grid: s_b in grid steps and phi (S - s_b), cut;
+// false where the exponents call for the FP64 form.
+RLT2_HD bool class_pool_fx(const double s[6], FxFactor phi, int64_t q[6], int64_t pool[6], uint32_t& emax) {
+  emax = 0;
   for (int b = 0; b < 6; ++b) {
-    const uint32_t a = fx_exp(D[b]), c = fx_exp(w[b]);
-    emax = emax > a ? emax : a;
-    emax = emax > c ? emax : c;
+    const uint32_t e = fx_exp(s[b]);
+    emax = emax > e ? emax : e;
   }
   if (emax < kFxExpLow || emax > kFxExpHigh) return false;
-  int64_t s[6], q[6], S = 0;
+  int64_t S = 0;
   for (int b = 0; b < 6; ++b) {
-    q[b] = fx_align(w[b], emax);
-    s[b] = fx_align(D[b], emax) - q[b];
-    S += s[b];
+    q[b] = fx_align(s[b], emax);
+    S += q[b];
   }
-  for (int b = 0; b < 6; ++b) D[b] = fx_unalign(q[b] + fx_scale(phi, S - s[b]), emax);
+  for (int b = 0; b < 6; ++b) pool[b] = fx_scale(phi, S - q[b]);
+  return true;
+}
+
+// The move of one class, in place on D, s_b = (D_b - xi_b) - psi_b; false (D
+// untouched) where the exponents call for the FP64 form.
+RLT2_HD bool pool_class_fx(double D[6], const double s[6], FxFactor phi) {
+  int64_t q[6], pool[6];
+  uint32_t emax;
+  if (!class_pool_fx(s, phi, q, pool, emax)) return false;
+  for (int b = 0; b < 6; ++b) D[b] += fx_unalign(pool[b] - q[b], emax);
+  return true;
+}
+
+// The same move for a host program that holds the sums w_b = xi_b + psi_b:
+// D'_b = w_b + phi (S - s_b), s_b = D_b - w_b, so that the result keeps what the
+// sum has where s_b cancels most of D_b.  A class without slack stays as it is.
+inline bool move_class_fx(double D[6], const double w[6], FxFactor phi) {
+  double s[6];
+  int64_t q[6], pool[6];
+  uint32_t emax;
+  bool rest = true, zero = true;
+  for (int b = 0; b < 6; ++b) {
+    s[b] = D[b] - w[b];
+    rest = rest && s[b] == 0.0;
+    zero = zero && D[b] == 0.0;
+  }
+  if (rest && !zero) return true;
+  if (!class_pool_fx(s, phi, q, pool, emax)) return false;
+  for (int b = 0; b < 6; ++b) D[b] = w[b] + fx_unalign(pool[b], emax);
   return true;
 }
 
