@@ -621,12 +621,15 @@ cudaError_t gemm(bool ta, bool tb, int epi, int M, int N, int K, const bf16* A, 
     u.bias = bias;
     u.mask = mask;
     u.err = err;
-    // a K split over the batch (weight gradients): about one CTA per SM, at least
-    // 256 rows each (a gradient call of 8,192 rows 144 -> 130 us, of 200,000 579
-    // -> 542; two CTAs per SM 552, splits of 512 rows 144)
-    const int blocks = ((M + 127) / 128) * ((N + 127) / 128);
-    const int tsplits = splits > 1 ? std::max(1, std::min(152 / blocks, K / 256)) : 1;
-    return umma_gemm(u, tsplits, s);
+    int parts = 1;
+    if (splits > 1) {  // weight gradients
+      int dev = 0, sms = 0;
+      cudaError_t e = cudaGetDevice(&dev);
+      if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+      if (e != cudaSuccess) return e;
+      parts = wgrad_parts(K, ((M + 127) / 128) * ((N + 127) / 128), sms);
+    }
+    return umma_gemm(u, parts, s);
   }
   const int kps = ((K / splits + BK - 1) / BK) * BK;
   dim3 grid(N / BN, M / BM, (K + kps - 1) / kps);
