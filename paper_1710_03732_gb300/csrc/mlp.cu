@@ -20,6 +20,7 @@
 // significand on the integer pipe) because FP64 is GB300's scarce resource.
 #include <cuda_bf16.h>
 
+#include <cfloat>
 #include <cmath>
 #include <cstdint>
 #include <cstring>
@@ -96,7 +97,7 @@ __device__ __forceinline__ unsigned sort_rows(unsigned v, const SortFlips& x) {
   }
   return v ^ x.f[s];
 }
-// The same on floats, one row (scaled rows that overflow FP32).
+// The same on floats, one row (rows whose scale or its inverse overflows FP32).
 __device__ __forceinline__ float sort_row(float v, int lane) {
 #pragma unroll
   for (int k = 2; k <= 32; k <<= 1) {
@@ -150,6 +151,9 @@ __global__ void __launch_bounds__(kFeatWarps * 32) k_features(long long ntiles, 
     rmax = __uint_as_float(__reduce_max_sync(kFull, __float_as_uint(rmax)));  // non-negative: ordered as integers
     const float s = rmax > 0.0f ? rmax : 1.0f;
     const float inv = __fdiv_rn(1.0f, s);
+    // s or 1/s beyond FP32: 0 times infinity makes NaN, whose place among the keys
+    // is not the one that fminf and fmaxf give it
+    const bool plain = s <= FLT_MAX && inv <= FLT_MAX;
     if (lane == 0 && scale) scale[t] = s;
     const float pv = prev_u ? __fmul_rn(f32_trunc(pd), inv) : 0.0f;  // row `lane`'s scaled previous dual
     unsigned* xr = reinterpret_cast<unsigned*>(X + t * m * kInPad) + (lane >> 1);
@@ -159,7 +163,7 @@ __global__ void __launch_bounds__(kFeatWarps * 32) k_features(long long ntiles, 
       const float va = col ? __fmul_rn(__fsub_rn(sm[i * m + lane], cmin), inv) : INFINITY;
       const float vb = col ? __fmul_rn(__fsub_rn(sm[i1 * m + lane], cmin), inv) : INFINITY;
       unsigned w;
-      if (s <= 3.402823466e38f) {
+      if (plain) {
         const __nv_bfloat162 r = __floats2bfloat162_rn(va, vb);
         w = sort_rows<W>(*reinterpret_cast<const unsigned*>(&r), flips);
       } else {
