@@ -402,15 +402,15 @@ struct LapPlan {
   size_t smem = 0;
 };
 
-// Launch configuration, kept per device and set once per (device, size, group,
-// warps) under g_cfg_mu: contexts may be created and used from different host
+// Launch configuration, kept per device and set once per (device, size; for nodes
+// also lanes and warps) under g_cfg_mu: contexts may be created and used from different host
 // threads and on different devices.  Like every per-device cache of the library
 // it is not valid across a cudaDeviceReset.
 static std::mutex g_cfg_mu;
 constexpr int kMaxCfgDevices = 64;
 struct LapDevCfg {
   int sms = 0;                        // multiprocessors of the device
-  LapPlan plan[33][3][2][kForms];     // for (m, G, warps per block, form)
+  LapPlan plan[33][kForms];           // k_lap, for (m, form)
   int occ_nodes[33][3][2] = {};
   bool attr[3] = {};                  // dynamic shared-memory attribute set (k_lap, per G)
   bool attr_nodes[3] = {};            // the same for k_lap_nodes
@@ -429,11 +429,13 @@ static cudaError_t current_cfg(LapDevCfg** out) {
   return cudaSuccess;
 }
 
-// Every form of (G, m, wpb).  A fixed-point form takes two tile buffers per
+// Every form of size m.  A fixed-point form takes two tile buffers per
 // warp unless one tile alone lets more warps onto an SM: m = 28 (16 -> 32
 // warps), not m = 18 (32 either way).
-static cudaError_t prepare_one(LapDevCfg& cfg, int G, int m, int wpb) {
-  LapPlan* plan = cfg.plan[m][gidx(G)][wpb == 4 ? 0 : 1];
+static cudaError_t prepare_one(LapDevCfg& cfg, int m) {
+  const int G = default_group(m);
+  constexpr int wpb = kMaxWarpsPerBlock;
+  LapPlan* plan = cfg.plan[m];
   if (plan[kForms - 1].occ > 0) return cudaSuccess;
   cudaError_t e;
   const int cap = (int)(warp_smem_bytes_async(32, 32) * kMaxWarpsPerBlock);
@@ -467,37 +469,34 @@ static cudaError_t prepare_one(LapDevCfg& cfg, int G, int m, int wpb) {
 
 // The plan of an m-column LAP launch on the current device (configured on
 // first use), *cap its resident block count.
-static cudaError_t prepare_plan(int m, int group, int warps_per_block, int form, LapPlan* plan, long long* cap) {
+static cudaError_t prepare_plan(int m, int form, LapPlan* plan, long long* cap) {
   if (m < 1 || m > 32) return cudaErrorInvalidValue;
-  const int G = group ? group : default_group(m);
-  const int wpb = warps_per_block ? warps_per_block : kMaxWarpsPerBlock;
-  if (G < m || (G != 8 && G != 16 && G != 32) || (wpb != 4 && wpb != 8)) return cudaErrorInvalidValue;
   std::lock_guard<std::mutex> lock(g_cfg_mu);
   LapDevCfg* cfg = nullptr;
   cudaError_t e = current_cfg(&cfg);
   if (e != cudaSuccess) return e;
-  if ((e = prepare_one(*cfg, G, m, wpb)) != cudaSuccess) return e;
-  *plan = cfg->plan[m][gidx(G)][wpb == 4 ? 0 : 1][form];
+  if ((e = prepare_one(*cfg, m)) != cudaSuccess) return e;
+  *plan = cfg->plan[m][form];
   *cap = (long long)cfg->sms * plan->occ;
   return cudaSuccess;
 }
 
-cudaError_t prepare_lap(int m, int group, int warps_per_block) {
+cudaError_t prepare_lap(int m) {
   LapPlan plan;
   long long cap = 0;
-  return prepare_plan(m, group, warps_per_block, 0, &plan, &cap);
+  return prepare_plan(m, 0, &plan, &cap);
 }
 
 cudaError_t launch_lap(const LapArgs& a, cudaStream_t s) {
   if (a.batch <= 0) return cudaSuccess;
-  const int G = a.group ? a.group : default_group(a.m);
-  const int wpb = a.warps_per_block ? a.warps_per_block : kMaxWarpsPerBlock;
+  const int G = default_group(a.m);
+  constexpr int wpb = kMaxWarpsPerBlock;
   if (a.Badd || a.pi) return cudaErrorInvalidValue;  // launch_lap_blocks
   // a cold fixed-point launch reduces the rows first (the same canonical result)
   const int form = lap_form(a);
   LapPlan plan;
   long long cap = 0;
-  cudaError_t e = prepare_plan(a.m, G, wpb, form, &plan, &cap);
+  cudaError_t e = prepare_plan(a.m, form, &plan, &cap);
   if (e != cudaSuccess) return e;
   LapArgs b = a;
   b.prefetch = plan.prefetch;
@@ -523,9 +522,8 @@ cudaError_t launch_lap(const LapArgs& a, cudaStream_t s) {
 bool lap_wants_queue(long long batch, int m) {
   LapPlan plan;
   long long cap = 0;
-  const int G = default_group(m);
-  if (prepare_plan(m, G, kMaxWarpsPerBlock, 1, &plan, &cap) != cudaSuccess) return false;
-  return batch > cap * kMaxWarpsPerBlock * (32 / G);
+  if (prepare_plan(m, 1, &plan, &cap) != cudaSuccess) return false;
+  return batch > cap * kMaxWarpsPerBlock * (32 / default_group(m));
 }
 
 // ---------------------------------------------------------------------------

@@ -181,7 +181,6 @@ struct Wave {
   int max_m[kStages] = {0, 0, 0, 0};
   int max_trips = 0;
   int max_T = 0;
-  int max_n = 0;
   std::vector<int> zm;     // Z-LAP size of each sorted Z item
   std::vector<ZRun> runs;  // the Z stages' launches
 };
@@ -376,7 +375,6 @@ void add_node(Wave& w, WaveHost& h, int j, const IterView& v, const rlt2_params&
   h.fin[j] = make_fin(v);
   w.max_trips = std::max(w.max_trips, h.mzb[j]);
   w.max_T = std::max(w.max_T, (int)v.T);
-  w.max_n = std::max(w.max_n, nr);
 }
 
 // The Z stages' items sorted by LAP size (stable: node order within a size).

@@ -99,14 +99,12 @@ struct LapArgs {
   int dual_mode;             // 0 raw (FP64), 1 canonical (fixed point), 2 canonical (FP64)
   unsigned long long* stats; // nullable, [0] += augmentations, [1] += relaxations
   const int* skip;           // nullable: kernel does nothing when *skip != 0
-  int group;                 // lanes per LAP (8, 16 or 32); 0 = smallest that fits m
-  int warps_per_block;       // 4 or 8; 0 = 8
   const int* map;            // nullable: LAP b works on slot map[b] of every array (a subset of tiles)
   long long fixed_part;      // set by launch_lap: LAPs below this are taken in a fixed stride, the rest from head
   int prefetch;              // set by launch_lap (2: its one-tile form): the fixed-point form without Badd and pi stages
                              // the next tile by cp.async while it solves the current one
-  unsigned long long* head;  // nullable: device counter of the prefetching form's LAP queue
-                             // (launch_lap zeroes it on the stream before the launch)
+  unsigned long long* head;  // nullable: device counter of the fixed-point form's LAP queue, zeroed by
+                             // launch_lap on the stream unless head_zeroed
   int wide;                  // set by launch_lap: tiles start on 16-byte boundaries (m even, A aligned)
   int dependent;             // launched as a programmatic dependent (see launch_dependent)
   int head_zeroed;           // an earlier launch on the stream has zeroed *head: no memset
@@ -187,13 +185,12 @@ int default_group(int m);
 
 // Configure the LAP kernel for size m (shared-memory limit, occupancy); call
 // outside stream capture before the first launch of that size.
-cudaError_t prepare_lap(int m, int group = 0, int warps_per_block = 0);
+cudaError_t prepare_lap(int m);
 
 // Enqueue the batched LAP kernel (grid sized for the device); returns the CUDA error.
 // Without Badd and pi.
 cudaError_t launch_lap(const LapArgs& a, cudaStream_t s);
-// One block per LAP, with Badd and pi (the Y and X stages; head, group and
-// warps_per_block unused).
+// One block per LAP, with Badd and pi (the Y and X stages; head unused).
 cudaError_t launch_lap_blocks(const LapArgs& a, cudaStream_t s);
 
 // Whether a fixed-point batch of the default shape is more than its resident
