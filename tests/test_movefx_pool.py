@@ -140,7 +140,7 @@ def _members(n):
 
 @pytest.mark.gpu
 @pytest.mark.parametrize("spread", [0, 3, 60])
-@pytest.mark.parametrize("n", [3, 4, 5, 6, 8, 9, 11, 13])
+@pytest.mark.parametrize("n", [3, 4, 5, 6, 8, 9, 11, 13, 15])
 def test_device_move_equals_host_move(move, n, spread):
     from paper_1710_03732_gb300 import instances as I
     from paper_1710_03732_gb300 import rlt2 as R
