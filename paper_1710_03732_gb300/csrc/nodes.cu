@@ -38,19 +38,22 @@ __global__ void k_move_y_nodes(const MoveYArgs* nodes) {
   else move_y_range(a, start, stride);
 }
 
-// blockIdx.x = triple, blockIdx.y = node; a block goes through the triple's warps,
-// so that the node's arguments, read from global memory, cost one latency per
-// triple and nodes smaller than the largest leave few empty blocks (64 nodes of
-// residual 14 to 18: 350 -> 341 ms for 20 iterations against a block per eight
-// warps).  FIXED: the nodes whose own parameters give the integer form, else the
-// others; a node moves as it would alone, whatever shares its wave.
+// blockIdx.x = triple, blockIdx.y = node, the triple's warps shared out over the
+// gridDim.z blocks of a triple (Wave::slices).  Where the wave's triples alone fill
+// the GPU that is one block, which reads the node's arguments from global memory
+// once per triple and leaves few empty blocks for nodes smaller than the largest
+// (64 nodes of residual 14 to 18, 20 iterations: 308 ms against 324 with a block
+// per eight warps); a wave of a few small nodes would wait for the block's turns
+// (one node of residual 9, per iteration: 73.7 us, 69.4 with three blocks).  FIXED:
+// the nodes whose own parameters give the integer form, else the others; a node
+// moves as it would alone, whatever shares its wave.
 template <bool FIXED>
 __global__ void __launch_bounds__(256, 4) k_move_z_nodes(const MoveZArgs* nodes, const int* ntrips) {
   const MoveZArgs& a = nodes[blockIdx.y];
   if ((int)blockIdx.x >= ntrips[blockIdx.y] || (a.fixed != 0) != FIXED) return;
   if (!a.sc->have_snap || a.sc->done) return;
 #pragma unroll 1
-  for (int w = threadIdx.x >> 5; w < class_warps(a.n); w += 8)
+  for (int w = blockIdx.z * 8 + (threadIdx.x >> 5); w < class_warps(a.n); w += 8 * gridDim.z)
     move_z_warp<FIXED>(a, blockIdx.x, w, threadIdx.x & 31);
 }
 
@@ -58,7 +61,8 @@ __global__ void __launch_bounds__(256, 4) k_phase2_nodes(const Phase2Args* nodes
   const Phase2Args& a = nodes[blockIdx.y];
   if ((int)blockIdx.x >= ntrips[blockIdx.y] || a.sc->done) return;
 #pragma unroll 1
-  for (int w = threadIdx.x >> 5; w < class_warps(a.n); w += 8) phase2_warp(a, blockIdx.x, w, threadIdx.x & 31);
+  for (int w = blockIdx.z * 8 + (threadIdx.x >> 5); w < class_warps(a.n); w += 8 * gridDim.z)
+    phase2_warp(a, blockIdx.x, w, threadIdx.x & 31);
 }
 
 __global__ void __launch_bounds__(256) k_finalize_nodes(const FinArgs* nodes) {
@@ -180,6 +184,7 @@ struct Wave {
   long long total[kStages] = {0, 0, 0, 0};
   int max_m[kStages] = {0, 0, 0, 0};
   int max_trips = 0;
+  int slices = 1;  // blocks per triple of the class moves
   int max_T = 0;
   std::vector<int> zm;     // Z-LAP size of each sorted Z item
   std::vector<ZRun> runs;  // the Z stages' launches
@@ -253,7 +258,7 @@ cudaError_t enqueue_wave_iteration(const Wave& w, const WaveDev& d, int dual_mod
     k_move_y_nodes<<<dim3(bx, w.nn), 256, 0, s>>>(d.my);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
-  const dim3 class_grid(w.max_trips, w.nn);
+  const dim3 class_grid(w.max_trips, w.nn, w.slices);
   if (w.moves[1]) k_move_z_nodes<true><<<class_grid, 256, 0, s>>>(d.mz, d.mz_trips);
   if (w.moves[0]) k_move_z_nodes<false><<<class_grid, 256, 0, s>>>(d.mz, d.mz_trips);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
@@ -375,6 +380,23 @@ void add_node(Wave& w, WaveHost& h, int j, const IterView& v, const rlt2_params&
   h.fin[j] = make_fin(v);
   w.max_trips = std::max(w.max_trips, h.mzb[j]);
   w.max_T = std::max(w.max_T, (int)v.T);
+}
+
+// Wave::slices: so many that the triples' blocks fill the four that an SM holds, at
+// most one per eight warps of the largest node's triples.
+cudaError_t plan_classes(Wave& w, const WaveHost& h) {
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  long long trips = 0;
+  int most = 1;
+  for (int j = 0; j < w.nn; ++j) {
+    trips += h.mzb[j];
+    most = std::max(most, (class_warps(h.mz[j].n) + 7) / 8);
+  }
+  w.slices = (int)std::min<long long>(most, (4ll * sms + trips - 1) / trips);
+  return cudaSuccess;
 }
 
 // The Z stages' items sorted by LAP size (stable: node order within a size).
@@ -540,6 +562,7 @@ cudaError_t iterate_views(const IterView* views, int nn, const rlt2_params& prm,
   WaveHost h(nn);
   for (int j = 0; j < nn; ++j) add_node(w, h, j, views[j], prm);
   sort_z(w, h);
+  if ((e = plan_classes(w, h)) != cudaSuccess) return e;
   if ((e = upload_wave(w, h, d, s)) != cudaSuccess) return e;
   std::vector<cudaEvent_t> zev(2 * kMaxRuns, nullptr);
   for (cudaEvent_t& ev : zev)
@@ -738,6 +761,7 @@ extern "C" rlt2_status rlt2_bound_nodes(int n, const double* F, const double* D,
       add_node(w, hw, j, v, prm);
     }
     sort_z(w, hw);
+    CKN(plan_classes(w, hw));
     CKN(upload_wave(w, hw, d, s));
     // autotune the Z stage per LAP size on live iterations 2.. (iteration 1
     // has D^ = 0), then plan the Z launches
