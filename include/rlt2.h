@@ -115,12 +115,13 @@ typedef enum {
  *               the next solve as one launch, a tile's LAP starting once the
  *               move has finished every class of its facility pair (identical
  *               results; the FP64 move and the integer LAPs share the SMs);
- *               0 (default) = two launches.  On GB300 it pays for cold starts
- *               around n = 20 (13 % there) and loses elsewhere: the LAPs need
- *               the warp slots the move takes.  Not used with half_z or
- *               warm = 2, nor by rlt2_bound_nodes and the no-allocation entry
- *               point.  A pipelined wait that gives up (about a second; only a
- *               fault can cause it) stops the ascent and rlt2_iterate returns
+ *               0 (default) = two launches, which are faster on GB300 (n = 20
+ *               cold 1.15 against 1.42 ms per iteration, warm 0.68 against
+ *               1.13): the LAPs need the warp slots the move takes.  Not used
+ *               with half_z or warm = 2, nor by rlt2_bound_nodes and the
+ *               no-allocation entry point.  A pipelined wait that gives up
+ *               (about a second; only a fault can cause it) stops the ascent
+ *               and rlt2_iterate returns
  *               RLT2_ETIMEOUT. */
 typedef struct rlt2_params {
   double kz, ky, kx, phi_y;

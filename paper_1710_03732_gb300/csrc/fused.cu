@@ -1,8 +1,8 @@
 // The z move of an ascent step (Eq. 2.20-2.23, Section 3.3) and the Z-stage
 // LAPs of the next solve (Algorithm 1, Section 3.2) as one persistent launch.
 //
-// On GB300 the z move is bound by the FP64 pipe and the fixed-point Z-LAPs by
-// the integer ALU pipe.  Run back to back, each leaves the other pipe idle;
+// On GB300 the z move is bound by the FP64 pipe and the L2 tags and the fixed-point
+// Z-LAPs by the integer ALU pipe.  Run back to back, each leaves the other's idle;
 // here warps of the same SMs run both at once.  The data dependence between
 // them is narrow enough to allow it: the entries of Z tile (i,j,p,q) belong to
 // the classes {(i,p),(j,q),(k,r)}, which the move handles in its blocks
@@ -26,8 +26,10 @@
 // while theirs are not ready was tried: it starts the integer LAPs later and
 // was slower.)
 //
-// Used with rlt2_params.pipeline = 1, off by default: it pays for cold starts
-// near n = 20, while elsewhere the LAPs miss the warp slots the movers hold.
+// Used with rlt2_params.pipeline = 1, off by default: it is slower than the two
+// launches, whose kernels run with all of an SM's warps (per iteration, n = 20 cold
+// 1.42 against 1.15 ms, warm 1.13 against 0.68; n = 12 cold 130 against 93 us, warm
+// 115 against 66).
 #include <algorithm>
 #include <mutex>
 #include <vector>
@@ -44,9 +46,9 @@ constexpr int kPipeSpinLimit = 1 << 22;
 // The same limit in the failure-detection check, whose waits can never end.
 constexpr int kPipeCheckSpinLimit = 1 << 12;
 // Warps per block that run the move first (of kMaxWarpsPerBlock): 8 per SM keep
-// the integer move going through its load latencies, the other 24 run the
-// integer LAPs (n = 20 cold, warm per iteration: two 1.36, 1.08 ms, three 1.47,
-// 1.14, four 1.46, 1.12).
+// the move going through its load latencies, the other 24 run the integer LAPs
+// (n = 20 cold, warm per iteration: two 1.36, 1.08 ms, three 1.47, 1.14, four 1.46,
+// 1.12; 1.42, 1.13 with the move's slacks in FP64).
 constexpr int kMoveWarps = 2;
 
 // 64 registers: four blocks of eight warps per SM (80 unbounded: three)

@@ -38,9 +38,10 @@ constexpr int kIn = 34;      // features per row
 constexpr int kInPad = 64;   // padded input width (GEMM K)
 constexpr int kChunk = 1 << 18;  // rows per training chunk, and per inference chunk of widths other than 256
 // Rows per inference chunk of the 256-wide network (features, predictions and
-// scales only): 64 MB of features, which stay in L2.  At m = 18 a chunk is three
-// full waves of feature warps and 27 of the network's tiles, where 2^18 rows were
-// one and a half and 13.5: 144,400 tiles 1.10 -> 0.96 ms.
+// scales only): 64 MB of features, which stay in L2, and whole waves of the network's
+// tiles (27 of 152) where 2^18 rows were 13.5.  2.6 million rows, 2^18 against 2^19:
+// m = 4 993 -> 880 us, 8 949 -> 841, 12 998 -> 871, 18 1,105 -> 975, 24 1,192 -> 996,
+// 30 1,254 -> 1,035; 600,000 rows 7 to 13 % less; up to 2^18 rows the same.
 constexpr int kPredictChunk = 1 << 19;
 using bf16 = __nv_bfloat16;
 
@@ -677,7 +678,7 @@ cudaError_t backward(rlt2_mlp* m, const bf16* X, const float* T, long long rows,
   float* gw3 = gb2 + H;
   float* gb3 = gw3 + H;
   if ((e = forward(m, X, rows, nullptr, s)) != cudaSuccess) return e;
-  const int hblocks = (int)std::min<long long>(456, (rows + 15) / 16);  // three per SM
+  const int hblocks = (int)std::min<long long>(456, (rows + 15) / 16);  // three per SM of GB300
   if (H <= 256)
     k_head<8><<<hblocks, 256, 2 * H * sizeof(float), s>>>(rows, nvalid, H, m->H2, m->w3, m->b3, T, m->dH2, m->loss, gw3,
                                                          gb2, gb3);
